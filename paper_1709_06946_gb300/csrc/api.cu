@@ -15,6 +15,7 @@
 #include <new>
 
 #include "device_common.cuh"
+#include "krylov_math.cuh"
 #include "pse_internal.cuh"
 
 namespace pse {
@@ -935,6 +936,13 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
     k.l_cprev = (double *)A(sizeof(double) * ns * (size_t)L);
     k.l_c = (double *)A(sizeof(double) * ns * (size_t)L);
     k.l_work = (double *)A(sizeof(double) * ns * (size_t)(2 * L + L * L));
+    double *nodes = (double *)A(sizeof(double) * 2 * SQRT_NODES);
+    if (nodes) {
+      double h[2 * SQRT_NODES];
+      sqrt_nodes(SQRT_NODES, SQRT_WINDOW, h, h + SQRT_NODES);
+      PSE_CUDA_TRY(c, cudaMemcpy(nodes, h, sizeof(h), cudaMemcpyHostToDevice));
+    }
+    k.l_nodes = nodes;
     k.l_b0 = (double *)A(sizeof(double) * ns);
     k.l_err = (double *)A(sizeof(double) * ns);
     k.g_H = (double *)A(sizeof(double) * ns * (size_t)(M + 1) * M);

@@ -166,6 +166,7 @@ struct KDev {
   double *coef;
   int *active, *nrows, *iter, *flag;   // flag[0]: continue the loop
   double *l_alpha, *l_beta, *l_cprev, *l_c, *l_work, *l_b0, *l_err;
+  const double *l_nodes;               // nodes, then weights, of the rational square root
   int *l_it, *l_capped;
   double *g_H, *g_cs, *g_sn, *g_g, *g_beta, *g_rel;
   int *g_it, *g_capped;

@@ -568,6 +568,23 @@ int pse_internal_choose_tile(int Ng, int P, int ts, const int *caps, const int *
   return 0;
 }
 
+// c = T^{1/2} e_1 by the rational square root (as the Lanczos control kernel, node by
+// node).  Returns 1 when the spectrum of T leaves the window below the Gershgorin bound.
+int pse_internal_rational_sqrt_e1(int n, const double *d, const double *e, double *c) {
+  double s[pse::SQRT_NODES], w[pse::SQRT_NODES], hi = 0.0;
+  pse::sqrt_nodes(pse::SQRT_NODES, pse::SQRT_WINDOW, s, w);
+  for (int i = 0; i < n; ++i) hi = std::max(hi, d[i] + (i < n - 1 ? std::fabs(e[i]) : 0.0) + (i > 0 ? std::fabs(e[i - 1]) : 0.0));
+  std::vector<double> x(n), y(n, 0.0);
+  if (!pse::shifted_solve_e1(n, d, e, -hi / pse::SQRT_WINDOW, x.data(), 1)) return 1;
+  for (int k = 0; k < pse::SQRT_NODES; ++k) {
+    pse::shifted_solve_e1(n, d, e, hi * s[k], x.data(), 1);
+    for (int i = 0; i < n; ++i) y[i] += w[k] * x[i];
+  }
+  for (int i = 0; i < n; ++i)
+    c[i] = std::sqrt(hi) * (d[i] * y[i] + (i > 0 ? e[i - 1] * y[i - 1] : 0.0) + (i < n - 1 ? e[i] * y[i + 1] : 0.0));
+  return 0;
+}
+
 // c = T^{1/2} e_1 for the symmetric tridiagonal T (diagonal d, off-diagonal e).
 int pse_internal_tridiag_sqrt_e1(int n, const double *d, const double *e, double *c) {
   std::vector<double> dd(d, d + n), ee(e, e + (n > 1 ? n - 1 : 0)), Z;
