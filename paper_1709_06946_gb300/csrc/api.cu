@@ -98,8 +98,8 @@ cudaEvent_t prof_event(pse_ctx *c) {
   return e;
 }
 
-pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s) {
-  if (parts & PSE_PART_REAL) PSE_TRY(real_apply(c, vin, vout, mode, s));
+pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s, bool gathered) {
+  if (parts & PSE_PART_REAL) PSE_TRY(real_apply(c, vin, vout, mode, s, gathered));
   if (parts & PSE_PART_WAVE) PSE_TRY(wave_apply(c, vin, vout, mode, (parts & PSE_PART_REAL) != 0, s));
   if (!(parts & PSE_PART_ALL)) PSE_CUDA_TRY(c, cudaMemsetAsync(vout, 0, c->ts * 8 * (size_t)c->p.N, s));
   return PSE_OK;
@@ -131,7 +131,8 @@ pse_status set_all_active(pse_ctx *c, cudaStream_t s) {
   return PSE_OK;
 }
 
-// Runs `body` (one Krylov iteration, launched on the stream it is given) until
+// Runs `body` (one Krylov iteration, launched on the stream it is given, with the loop's
+// condition handle inside a capture) until
 // the control kernels clear the loop flag, at most `cap` times.  Outside a
 // capture this is a host loop that reads the flag (and the active set) after
 // every iteration; while the step is being captured it becomes a conditional
@@ -141,10 +142,9 @@ template <typename Body>
 pse_status krylov_loop(pse_ctx *c, int cap, cudaStream_t s, Body &&body) {
   if (!c->capturing) {
     for (int j = 0; j < cap; ++j) {
-      PSE_TRY(body(s));
-      kd_loop_end(c, cap, 0, 0, s);
-      PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_flag, c->kd.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-      PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_flag + 1, c->d_active, sizeof(int) * c->nsys, cudaMemcpyDeviceToHost, s));
+      PSE_TRY(body(s, 0, 0));
+      // the flag and, right behind it, the active set
+      PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_flag, c->kd.flag, sizeof(int) * (1 + c->nsys), cudaMemcpyDeviceToHost, s));
       PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
       c->h2d_pending = false;
       std::copy(c->h_flag + 1, c->h_flag + 1 + c->nsys, c->h_active.begin());
@@ -180,8 +180,7 @@ pse_status krylov_loop(pse_ctx *c, int cap, cudaStream_t s, Body &&body) {
   cudaGraph_t body_g = np.conditional.phGraph_out[0];
   PSE_CUDA_TRY(c, cudaStreamBeginCaptureToGraph(c->cap_stream, body_g, nullptr, nullptr, 0,
                                                 cudaStreamCaptureModeRelaxed));
-  pse_status st = body(c->cap_stream);
-  kd_loop_end(c, cap, h, 1, c->cap_stream);
+  pse_status st = body(c->cap_stream, h, 1);
   cudaGraph_t out_g = nullptr;
   cudaError_t e = cudaStreamEndCapture(c->cap_stream, &out_g);
   PSE_TRY(st);
@@ -189,31 +188,27 @@ pse_status krylov_loop(pse_ctx *c, int cap, cudaStream_t s, Body &&body) {
   return PSE_OK;
 }
 
-// Orthogonalise w against basis rows 0..j (j = the device iteration counter)
-// twice (classical Gram-Schmidt, FP64 coefficients), then |w|^2.
-pse_status cgs2(pse_ctx *c, void *w, cudaStream_t s) {
-  PSE_TRY(multidot_rows(c, c->d_basis, 1, w, CO_H1, s));
-  PSE_TRY(combine_sub_rows(c, w, c->d_basis, 1, CO_H1, s));
-  PSE_TRY(multidot_rows(c, c->d_basis, 1, w, CO_H2, s));
-  PSE_TRY(combine_sub_rows(c, w, c->d_basis, 1, CO_H2, s));
-  return multidot(c, w, 1, w, CO_NRM, s);
+// One recurrence from z (Lanczos) or b (GMRES) in the order of its basis rows; `apply`
+// launches w = A d_vin on the given stream.
+template <typename Apply>
+pse_status krylov(pse_ctx *c, const void *z, void *w, bool gm, int cap, cudaStream_t s, Apply &&apply) {
+  std::fill(c->h_active.begin(), c->h_active.end(), 1);
+  PSE_TRY(kr_start(c, z, gm, s));
+  PSE_TRY(kr_next(c, z, s));
+  PSE_TRY(krylov_loop(c, cap, s, [&](cudaStream_t t, cudaGraphConditionalHandle h, int graph) {
+    PSE_TRY(apply(t));
+    PSE_TRY(kr_step(c, w, gm, cap, h, graph, t));
+    return kr_next(c, w, t);
+  }));
+  return set_all_active(c, s);
 }
 
 // y = M_r^{1/2} z by Lanczos with full reorthogonalisation (Sec. 3.2), per
 // suspension, stopping rule and tridiagonal square root on the device.
 pse_status lanczos(pse_ctx *c, const void *z, void *y, void *w, cudaStream_t s) {
   const int cap = c->lanczos_max;
-  PSE_TRY(set_all_active(c, s));
-  PSE_TRY(multidot(c, z, 1, z, CO_NRM, s));
-  kd_lz_start(c, s);
-  PSE_TRY(vscale_row(c, c->d_basis, 0, z, c->d_vin, CO_FAC, s));
-  PSE_TRY(krylov_loop(c, cap, s, [&](cudaStream_t t) {
-    PSE_TRY(real_apply(c, c->d_vin, w, M_FULL, t));
-    PSE_TRY(cgs2(c, w, t));
-    kd_lz_step(c, t);
-    return vscale_row(c, c->d_basis, 1, w, c->d_vin, CO_FAC, t);
-  }));
-  PSE_TRY(set_all_active(c, s));
+  PSE_TRY(krylov(c, z, w, false, cap, s,
+                 [&](cudaStream_t t) { return real_apply(c, c->d_vin, w, M_FULL, t, true); }));
   return combine_set(c, y, c->d_basis, c->d_nrows, cap, CO_Y, s);
 }
 
@@ -221,17 +216,8 @@ pse_status lanczos(pse_ctx *c, const void *z, void *y, void *w, cudaStream_t s) 
 // suspension; stops at |r|/|b| <= tol.  b and x hold the stresslet in slots 3..7.
 pse_status gmres(pse_ctx *c, const void *b, void *x, void *w, cudaStream_t s) {
   const int cap = c->krylov_max;
-  PSE_TRY(set_all_active(c, s));
-  PSE_TRY(multidot(c, b, 1, b, CO_NRM, s));
-  kd_gm_start(c, s);
-  PSE_TRY(vscale_row(c, c->d_basis, 0, b, c->d_vin, CO_FAC, s));
-  PSE_TRY(krylov_loop(c, cap, s, [&](cudaStream_t t) {
-    PSE_TRY(mobility(c, c->d_vin, w, M_SE, PSE_PART_ALL, t));
-    PSE_TRY(cgs2(c, w, t));
-    kd_gm_step(c, t);
-    return vscale_row(c, c->d_basis, 1, w, c->d_vin, CO_FAC, t);
-  }));
-  PSE_TRY(set_all_active(c, s));
+  PSE_TRY(krylov(c, b, w, true, cap, s,
+                 [&](cudaStream_t t) { return mobility(c, c->d_vin, w, M_SE, PSE_PART_ALL, t, true); }));
   return combine_set(c, x, c->d_basis, c->d_nrows, cap, CO_Y, s);
 }
 
@@ -608,9 +594,20 @@ pse_status rfd_impl(pse_ctx *c, double *pos, const void *FP, double dt, double d
   return capped ? PSE_ERR_NOT_CONVERGED : PSE_OK;
 }
 
+// Vector elements per block for these suspensions (VEC_CHUNK_MAX ... VEC_CHUNK_MIN).
+int vec_chunk(const std::vector<Params> &ps) {
+  for (int ch = VEC_CHUNK_MAX; ch > VEC_CHUNK_MIN; ch /= 2) {
+    int64_t nb = 0;
+    for (const Params &q : ps) nb += ceil_div(8 * q.N, ch);
+    if (nb >= VEC_BLOCKS) return ch;
+  }
+  return VEC_CHUNK_MIN;
+}
+
 // Device memory of a handle before it is created (the admission estimate of a
 // serving loop); mirrors the allocations of create_group.
 int64_t estimate_bytes(const pse_ctx *c) {
+  const int chunk = vec_chunk(c->ps);
   const size_t ts = c->ts;
   int64_t Nt = 0, ntile = 0, ncell = 0, n3 = 0, nk = 0, nbr = 0, vblk = 0;
   for (const Params &q : c->ps) {
@@ -621,7 +618,7 @@ int64_t estimate_bytes(const pse_ctx *c) {
     nk += (int64_t)q.Ng * q.Ng * q.nkx;
     double mean = 4.0 / 3.0 * M_PI * q.rcut * q.rcut * q.rcut * q.N / q.V();
     nbr += (int64_t)std::max(8.0, std::ceil((1.4 * mean + 24) / 8.0) * 8.0) * q.N;
-    vblk += ceil_div(8 * q.N, VEC_CHUNK);
+    vblk += ceil_div(8 * q.N, chunk);
   }
   int rows = std::max(c->lanczos_max, c->krylov_max) + 1;
   int64_t b = 0;
@@ -751,6 +748,7 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
   c->n_cubic = 0;
   c->lattice = 0;
   for (int i = 0; i < 9; ++i) c->lattice |= o.deform[i] != 0.0 ? 1 : 0;
+  c->vchunk = vec_chunk(c->ps);
   std::vector<int64_t> p0(ns + 1, 0), k0(ns + 1, 0);
   std::vector<int> tile0(ns + 1, 0), blk0(ns + 1, 0);
   int64_t cell_tot = 0;
@@ -796,7 +794,7 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
     tile0[q + 1] = tile0[q] + p.ntile[0] * p.ntile[1] * p.ntile[2];
     cell_tot += (int64_t)p.nc * p.nc * p.nc;
     k0[q + 1] = k0[q] + (int64_t)p.Ng * p.Ng * p.nkx;
-    blk0[q + 1] = blk0[q] + (int)ceil_div(8 * p.N, VEC_CHUNK);
+    blk0[q + 1] = blk0[q] + (int)ceil_div(8 * p.N, c->vchunk);
   }
   if (cell_tot > 1500000000LL || (int64_t)tile0[ns] > 1500000000LL) {
     c->err = "too many cells or tiles";
@@ -853,7 +851,10 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
   c->d_k0 = (int64_t *)A(sizeof(int64_t) * (ns + 1));
   c->d_tile0 = (int *)A(sizeof(int) * (ns + 1));
   c->d_blk0 = (int *)A(sizeof(int) * (ns + 1));
-  c->d_active = (int *)A(sizeof(int) * ns);
+  c->kd.iter = (int *)A(sizeof(int) * (4 + (size_t)ns));  // iteration, -, -, loop flag, active set (read back together)
+  c->kd.flag = c->kd.iter + 3;
+  c->d_active = c->kd.iter + 4;
+  c->d_done = (int *)A(sizeof(int) * ((size_t)ns + 1));
   c->d_nrows = (int *)A(sizeof(int) * ns);
   c->kd.active = c->d_active;
   c->kd.nrows = c->d_nrows;
@@ -925,8 +926,6 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
     k.gmax = M;
     k.ltol = c->lanczos_tol;
     k.gtol = c->krylov_tol;
-    k.iter = (int *)A(sizeof(int) * 4);
-    k.flag = k.iter + 2;
     k.l_it = (int *)A(sizeof(int) * 2 * ns);   // l_it then l_capped (read back together)
     k.l_capped = k.l_it + ns;
     k.g_it = (int *)A(sizeof(int) * 2 * ns);   // g_it then g_capped
@@ -967,6 +966,7 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
   PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_flag, sizeof(int) * (1 + (size_t)ns)));
   PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_rng, 2 * sizeof(uint64_t)));
   PSE_CUDA_TRY(c, cudaMemset(c->kd.iter, 0, sizeof(int) * 4));
+  PSE_CUDA_TRY(c, cudaMemset(c->d_done, 0, sizeof(int) * ((size_t)ns + 1)));
   PSE_CUDA_TRY(c, cudaMemset(c->kd.l_it, 0, sizeof(int) * 2 * ns));
   PSE_CUDA_TRY(c, cudaMemset(c->kd.g_it, 0, sizeof(int) * 2 * ns));
   PSE_CUDA_TRY(c, cudaMemcpy(c->d_sys, c->hs.data(), sizeof(SysDev) * ns, cudaMemcpyHostToDevice));

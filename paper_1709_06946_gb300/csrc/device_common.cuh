@@ -14,12 +14,17 @@ __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + 
 
 // Persistent work loop: the CTA takes work items from the counter *queue (which
 // starts at zero) until `total` have been handed out; every thread of the CTA
-// calls f(item) for the same items, so f may use __syncthreads.
+// calls f(item) for the same items, so f may use __syncthreads.  Every CTA of the
+// (one-dimensional) grid takes exactly one number past the items; the last of them
+// resets the counter, so no launch clears it.
 template <class F>
 __device__ __forceinline__ void for_each_item(int *queue, int total, F &&f) {
   __shared__ int s_item;
   for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(queue, 1);
+    if (threadIdx.x == 0) {
+      s_item = atomicAdd(queue, 1);
+      if (s_item == total + (int)gridDim.x - 1) *queue = 0;
+    }
     __syncthreads();
     const int item = s_item;
     __syncthreads();

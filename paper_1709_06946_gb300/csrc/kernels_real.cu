@@ -224,7 +224,7 @@ void launch_real_m(pse_ctx *c, const RealArgs &a, const void *vin, void *vout, c
     static std::atomic<int> per_sm{0};
     const int64_t items = ceil_div(a.Ntot * G, 1024);
     unsigned grid = persistent_grid(c, kern, 1024, tab_bytes, items, per_sm);
-    int *q = next_queue(c, s);
+    int *q = next_queue(c);
     kern<<<grid, 1024, tab_bytes, s>>>(a, c->d_sys, c->d_p0, c->d_active, q, (int)items, c->d_nbr_start,
                                        (const typename V4<T>::t *)c->d_nbr_geo, (const T *)vin,
                                        (const T *)c->d_vcell, (T *)vout, (const T *)c->d_table);
@@ -237,7 +237,7 @@ void launch_real_m(pse_ctx *c, const RealArgs &a, const void *vin, void *vout, c
   if (sizeof(T) == 4 && MODE == M_SE) tab = c->d_table_e;
   if (sizeof(T) == 4 && (MODE == M_FSU || MODE == M_SU)) tab = c->d_table_u;
   unsigned grid = persistent_grid(c, kern, 256, 0, items, per_sm);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   kern<<<grid, 256, 0, s>>>(a, c->d_sys, c->d_p0, c->d_active, q, (int)items, c->d_nbr_start,
                             (const typename V4<T>::t *)c->d_nbr_geo, (const T *)vin, (const T *)c->d_vcell,
                             (T *)vout, (const T *)tab);
@@ -443,7 +443,7 @@ pse_status overlap_force(pse_ctx *c, double kspring, void *F, cudaStream_t s) {
 
 // vout = M_r vin for the current configuration (sorted order, [N][8]); rows of
 // inactive suspensions are left untouched.
-pse_status real_apply(pse_ctx *c, const void *vin, void *vout, int mode, cudaStream_t s) {
+pse_status real_apply(pse_ctx *c, const void *vin, void *vout, int mode, cudaStream_t s, bool gathered) {
   StageTimer timer(c, PSE_STAGE_REAL, s, mode);
   c->nlaunch += 1;
   RealArgs a;
@@ -454,14 +454,16 @@ pse_status real_apply(pse_ctx *c, const void *vin, void *vout, int mode, cudaStr
   a.inv_dr = 1.0 / c->table_dr;
   a.self_uf = c->self_uf;
   a.self_es = c->self_es;
-  c->nlaunch += 1;
+  if (!gathered) c->nlaunch += 1;
   const unsigned nb = (unsigned)ceil_div(c->p.N, 256);
   if (c->prec == PSE_MIXED) {
-    k_cell_gather<float><<<nb, 256, 0, s>>>(c->p.N, c->d_cell_list, (const float4 *)vin, (float4 *)c->d_vcell);
+    if (!gathered)
+      k_cell_gather<float><<<nb, 256, 0, s>>>(c->p.N, c->d_cell_list, (const float4 *)vin, (float4 *)c->d_vcell);
     launch_real<float>(c, a, vin, vout, mode, s);
   } else {
-    k_cell_gather<double><<<nb, 256, 0, s>>>(c->p.N, c->d_cell_list, (const double4_32a *)vin,
-                                             (double4_32a *)c->d_vcell);
+    if (!gathered)
+      k_cell_gather<double><<<nb, 256, 0, s>>>(c->p.N, c->d_cell_list, (const double4_32a *)vin,
+                                               (double4_32a *)c->d_vcell);
     launch_real<double>(c, a, vin, vout, mode, s);
   }
   PSE_CUDA_TRY(c, cudaGetLastError());
@@ -483,7 +485,7 @@ pse_status real_apply11(pse_ctx *c, const void *vin12, void *vout12, cudaStream_
   constexpr int G = 4;
   const int64_t items = ceil_div(a.Ntot * G, 256);
   const unsigned ng = (unsigned)ceil_div(12 * c->p.N, 256);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   if (c->prec == PSE_MIXED) {
     static std::atomic<int> per_sm{0};
     k_cell_gather12<float><<<ng, 256, 0, s>>>(c->p.N, c->d_cell_list, (const float *)vin12, (float *)c->d_vcell12);

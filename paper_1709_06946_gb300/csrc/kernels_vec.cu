@@ -11,11 +11,10 @@
 
 #include "device_common.cuh"
 #include "pse_internal.cuh"
+#include "vec_common.cuh"
 
 namespace pse {
 namespace {
-
-constexpr int DOT_NT = 256, DOT_ROWS = 8;
 
 template <typename T>
 __global__ void k_gather_in(int64_t N, const int *perm, const T *F, const T *S, T *out) {
@@ -101,154 +100,16 @@ __global__ void k_philox_w1(int64_t N, const int *perm, uint64_t seed, uint64_t 
   out[e] = z0;
 }
 
-// The chunked vector kernels: block b covers VEC_CHUNK elements of the [N][8]
-// vectors of one suspension (blocks of suspension s start at blk0[s]).
-struct Chunk {
-  int s;
-  int64_t beg, end;
-};
-__device__ __forceinline__ Chunk chunk_of(const SysDev *sys, const int *blk0, int nsys) {
-  Chunk ch;
-  ch.s = find_sys(blk0, nsys, blockIdx.x);
-  const SysDev &q = sys[ch.s];
-  ch.beg = 8 * q.p0 + (int64_t)(blockIdx.x - q.blk0) * VEC_CHUNK;
-  int64_t lim = 8 * (q.p0 + q.N);
-  ch.end = ch.beg + VEC_CHUNK < lim ? ch.beg + VEC_CHUNK : lim;
-  return ch;
-}
-
-struct VecArgs {
-  const SysDev *sys;
-  const int *blk0, *active;
-  int nsys;
-};
-
-// 16-byte vectors of the chunked kernels (a chunk holds a multiple of 8 elements
-// and starts 32-byte aligned): 4 floats or 2 doubles per access.
-template <typename T> struct V16;
-template <> struct V16<float> {
-  using t = float4;
-  static constexpr int n = 4;
-  static __device__ __forceinline__ void get(const float4 &v, float a[4]) {
-    a[0] = v.x;
-    a[1] = v.y;
-    a[2] = v.z;
-    a[3] = v.w;
-  }
-  static __device__ __forceinline__ float4 put(const float a[4]) { return make_float4(a[0], a[1], a[2], a[3]); }
-};
-template <> struct V16<double> {
-  using t = double2;
-  static constexpr int n = 2;
-  static __device__ __forceinline__ void get(const double2 &v, double a[2]) {
-    a[0] = v.x;
-    a[1] = v.y;
-  }
-  static __device__ __forceinline__ double2 put(const double a[2]) { return make_double2(a[0], a[1]); }
-};
-
-// acc[r] += rows[r0 + r] . w over the block's chunk, r < nr <= DOT_ROWS; each
-// thread keeps VEC_UNROLL independent 16-byte loads per row in flight
-constexpr int VEC_UNROLL = 4;
-template <typename T>
-__device__ __forceinline__ void chunk_dots(const Chunk &ch, const T *__restrict__ rows, int64_t stride, int r0, int nr,
-                                           const T *__restrict__ w, T acc[DOT_ROWS]) {
-  using V = V16<T>;
-  using VT = typename V::t;
-#pragma unroll
-  for (int r = 0; r < DOT_ROWS; ++r) acc[r] = 0;
-  const int64_t step = (int64_t)blockDim.x * V::n;
-  for (int64_t e0 = ch.beg + (int64_t)threadIdx.x * V::n; e0 < ch.end; e0 += VEC_UNROLL * step) {
-    T wv[VEC_UNROLL][V::n];
-#pragma unroll
-    for (int u = 0; u < VEC_UNROLL; ++u) {
-      const int64_t e = e0 + u * step;
-      if (e < ch.end) V::get(*(const VT *)(w + e), wv[u]);
-      else
-#pragma unroll
-        for (int i = 0; i < V::n; ++i) wv[u][i] = 0;
-    }
-#pragma unroll
-    for (int r = 0; r < DOT_ROWS; ++r)
-      if (r < nr) {
-        const T *row = rows + (r0 + r) * stride;
-        T x[VEC_UNROLL][V::n];
-#pragma unroll
-        for (int u = 0; u < VEC_UNROLL; ++u) {
-          const int64_t e = e0 + u * step;
-          if (e < ch.end) V::get(*(const VT *)(row + e), x[u]);
-          else
-#pragma unroll
-            for (int i = 0; i < V::n; ++i) x[u][i] = 0;
-        }
-#pragma unroll
-        for (int u = 0; u < VEC_UNROLL; ++u)
-#pragma unroll
-          for (int i = 0; i < V::n; ++i) acc[r] += x[u][i] * wv[u][i];
-      }
-  }
-}
-
-// partial[b * pstride + r0 + r] = block sum of acc[r] (FP64 across threads), r < nr
-template <typename T>
-__device__ __forceinline__ void block_sums(const T acc[DOT_ROWS], int nr, double *partial, int pstride, int r0,
-                                           double red[DOT_ROWS][DOT_NT / 32]) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int r = 0; r < DOT_ROWS; ++r) {
-    if (r < nr) {
-      double v = (double)acc[r];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[r][wid] = v;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < nr) {
-    double sum = 0;
-    for (int k = 0; k < DOT_NT / 32; ++k) sum += red[threadIdx.x][k];
-    partial[(size_t)blockIdx.x * pstride + r0 + threadIdx.x] = sum;
-  }
-  __syncthreads();
-}
-
-// partial[b][r] = sum over block b's chunk of rows[r] . w   (r < nrows <= DOT_ROWS)
-template <typename T>
-__global__ void k_multidot(VecArgs va, const T *__restrict__ rows, int64_t stride, int nrows,
-                           const T *__restrict__ w, double *partial) {
-  __shared__ double red[DOT_ROWS][DOT_NT / 32];
-  const Chunk ch = chunk_of(va.sys, va.blk0, va.nsys);
-  if (!va.active[ch.s]) return;
-  T acc[DOT_ROWS];
-  chunk_dots(ch, rows, stride, 0, nrows, w, acc);
-  block_sums(acc, nrows, partial, DOT_ROWS, 0, red);
-}
-
-// out[s * COEF_STRIDE + r] = sum of the partials of suspension s (one block per suspension).
-__global__ void k_dot_final(VecArgs va, const double *partial, int nrows, double *out) {
-  const int s = blockIdx.x;
-  if (!va.active[s]) return;
-  int r = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (r >= nrows) return;
-  const int b0 = va.blk0[s], b1 = va.blk0[s + 1];
-  double sum = 0;
-  for (int b = b0 + lane; b < b1; b += 32) sum += partial[(size_t)b * DOT_ROWS + r];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (lane == 0) out[(size_t)s * COEF_STRIDE + r] = sum;
-}
-
 // w[e] = (SET ? 0 : w[e]) + sgn * sum_r coef[s][r] rows[r][e], r < nrows (or nrows_s[s])
 template <typename T, bool SET>
 __global__ void k_combine(VecArgs va, T *w, const T *__restrict__ rows, int64_t stride, int nrows,
-                          const int *__restrict__ nrows_s, const double *__restrict__ coef, T sgn,
-                          const int *__restrict__ nrows_dev = nullptr, int add = 0) {
+                          const int *__restrict__ nrows_s, const double *__restrict__ coef, T sgn) {
   using V = V16<T>;
   using VT = typename V::t;
   __shared__ T cs[MAX_ROWS];
-  const Chunk ch = chunk_of(va.sys, va.blk0, va.nsys);
+  const Chunk ch = chunk_of(va);
   if (!va.active[ch.s]) return;
-  int nr = nrows_dev ? min(*nrows_dev + add, MAX_ROWS) : nrows;
+  int nr = nrows;
   if (nrows_s) nr = min(nr, nrows_s[ch.s]);
   const double *cf = coef + (size_t)ch.s * COEF_STRIDE;
   for (int r = threadIdx.x; r < nr; r += blockDim.x) cs[r] = (T)cf[r];
@@ -294,65 +155,12 @@ __global__ void k_combine(VecArgs va, T *w, const T *__restrict__ rows, int64_t 
   }
 }
 
-// partial[b][r] = sum over block b's chunk of rows[r] . w for r < *nrows_dev + add
-// (at most MAX_ROWS), eight rows per pass over w.
-template <typename T>
-__global__ void k_multidot_rows(VecArgs va, const T *__restrict__ rows, int64_t stride, const int *nrows_dev, int add,
-                                const T *__restrict__ w, double *partial) {
-  __shared__ double red[DOT_ROWS][DOT_NT / 32];
-  const Chunk ch = chunk_of(va.sys, va.blk0, va.nsys);
-  if (!va.active[ch.s]) return;
-  const int nrows = min(*nrows_dev + add, MAX_ROWS);
-  for (int r0 = 0; r0 < nrows; r0 += DOT_ROWS) {
-    const int nr = min(DOT_ROWS, nrows - r0);
-    T acc[DOT_ROWS];
-    chunk_dots(ch, rows, stride, r0, nr, w, acc);
-    block_sums(acc, nr, partial, MAX_ROWS, r0, red);
-  }
-}
-
-// out[s * COEF_STRIDE + r] = sum of suspension s's partials, r < *nrows_dev + add (one block per suspension).
-__global__ void k_dot_final_rows(VecArgs va, const double *partial, const int *nrows_dev, int add, double *out) {
-  const int s = blockIdx.x;
-  if (!va.active[s]) return;
-  const int nrows = min(*nrows_dev + add, MAX_ROWS);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int b0 = va.blk0[s], b1 = va.blk0[s + 1];
-  for (int r = wid; r < nrows; r += nw) {
-    double sum = 0;
-    for (int b = b0 + lane; b < b1; b += 32) sum += partial[(size_t)b * MAX_ROWS + r];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) out[(size_t)s * COEF_STRIDE + r] = sum;
-  }
-}
-
-// basis row *iter + delta (and vin when given) = coef[s][0] * src
-template <typename T>
-__global__ void k_vscale_row(VecArgs va, T *basis, int64_t stride, const int *iter, int delta, const T *src, T *vin,
-                             const double *__restrict__ coef) {
-  using V = V16<T>;
-  using VT = typename V::t;
-  const Chunk ch = chunk_of(va.sys, va.blk0, va.nsys);
-  if (!va.active[ch.s]) return;
-  const T f = (T)coef[(size_t)ch.s * COEF_STRIDE];
-  T *dst = basis + (int64_t)(*iter + delta) * stride;
-  for (int64_t e = ch.beg + (int64_t)threadIdx.x * V::n; e < ch.end; e += (int64_t)blockDim.x * V::n) {
-    T x[V::n];
-    V::get(*(const VT *)(src + e), x);
-#pragma unroll
-    for (int i = 0; i < V::n; ++i) x[i] *= f;
-    *(VT *)(dst + e) = V::put(x);
-    if (vin) *(VT *)(vin + e) = V::put(x);
-  }
-}
-
 // dst = f * src with f = a, or f = coef[s][0] per suspension when coef is given
 template <typename T>
 __global__ void k_vscale(VecArgs va, T *dst, const T *src, T a, const double *__restrict__ coef) {
   using V = V16<T>;
   using VT = typename V::t;
-  const Chunk ch = chunk_of(va.sys, va.blk0, va.nsys);
+  const Chunk ch = chunk_of(va);
   if (!va.active[ch.s]) return;
   const T f = coef ? (T)coef[(size_t)ch.s * COEF_STRIDE] : a;
   for (int64_t e = ch.beg + (int64_t)threadIdx.x * V::n; e < ch.end; e += (int64_t)blockDim.x * V::n) {
@@ -465,18 +273,7 @@ __global__ void k_finite(const T *p, int64_t n, int *bad) {
     }
 }
 
-__global__ void k_clear(int *q) { *q = 0; }
-
 unsigned grid_for(int64_t n, int nt = 256) { return (unsigned)ceil_div(n, nt); }
-
-VecArgs vec_args(const pse_ctx *c) {
-  VecArgs v;
-  v.sys = c->d_sys;
-  v.blk0 = c->d_blk0;
-  v.active = c->d_active;
-  v.nsys = c->nsys;
-  return v;
-}
 
 }  // namespace
 
@@ -489,11 +286,7 @@ VecArgs vec_args(const pse_ctx *c) {
     }                               \
   } while (0)
 
-int *next_queue(pse_ctx *c, cudaStream_t s) {
-  int *q = c->d_queue + (c->queue_slot++ & 63);
-  k_clear<<<1, 1, 0, s>>>(q);
-  return q;
-}
+int *next_queue(pse_ctx *c) { return c->d_queue + (c->queue_slot++ & 63); }
 
 pse_status gather_in(pse_ctx *c, const void *F, const void *S, void *vout, cudaStream_t s) {
   StageTimer timer(c, PSE_STAGE_VECTOR, s);
@@ -562,57 +355,6 @@ pse_status philox_w1(pse_ctx *c, uint64_t seed, uint64_t counter, void *vout, cu
   const uint64_t *rng = c->capturing ? c->d_rng : nullptr;
   DISPATCH(c, (k_philox_w1<float><<<grid_for(8 * N), 256, 0, s>>>(N, c->d_perm, seed, counter, rng, (float *)vout)),
            (k_philox_w1<double><<<grid_for(8 * N), 256, 0, s>>>(N, c->d_perm, seed, counter, rng, (double *)vout)));
-  PSE_CUDA_TRY(c, cudaGetLastError());
-  return PSE_OK;
-}
-
-// coef[s][off + r] = rows[r] . w over suspension s, for r < nrows (rows of length 8N, contiguous).
-pse_status multidot(pse_ctx *c, const void *rows, int nrows, const void *w, int off, cudaStream_t s) {
-  StageTimer timer(c, PSE_STAGE_VECTOR, s);
-  const int64_t n = 8 * c->p.N;
-  const unsigned nb = (unsigned)c->nvblk;
-  VecArgs va = vec_args(c);
-  for (int r0 = 0; r0 < nrows; r0 += DOT_ROWS) {
-    int nr = std::min(DOT_ROWS, nrows - r0);
-    DISPATCH(c, (k_multidot<float><<<nb, DOT_NT, 0, s>>>(va, (const float *)rows + (size_t)r0 * n, n, nr, (const float *)w, c->d_dots)),
-             (k_multidot<double><<<nb, DOT_NT, 0, s>>>(va, (const double *)rows + (size_t)r0 * n, n, nr, (const double *)w, c->d_dots)));
-    k_dot_final<<<c->nsys, 32 * DOT_ROWS, 0, s>>>(va, c->d_dots, nr, c->d_coef + off + r0);
-    c->nlaunch += 2;
-  }
-  PSE_CUDA_TRY(c, cudaGetLastError());
-  return PSE_OK;
-}
-
-pse_status multidot_rows(pse_ctx *c, const void *rows, int add, const void *w, int off, cudaStream_t s) {
-  StageTimer timer(c, PSE_STAGE_VECTOR, s);
-  const int64_t n = 8 * c->p.N;
-  VecArgs va = vec_args(c);
-  c->nlaunch += 2;
-  DISPATCH(c, (k_multidot_rows<float><<<(unsigned)c->nvblk, DOT_NT, 0, s>>>(va, (const float *)rows, n, c->kd.iter, add, (const float *)w, c->d_dots)),
-           (k_multidot_rows<double><<<(unsigned)c->nvblk, DOT_NT, 0, s>>>(va, (const double *)rows, n, c->kd.iter, add, (const double *)w, c->d_dots)));
-  k_dot_final_rows<<<c->nsys, 256, 0, s>>>(va, c->d_dots, c->kd.iter, add, c->d_coef + off);
-  PSE_CUDA_TRY(c, cudaGetLastError());
-  return PSE_OK;
-}
-
-pse_status combine_sub_rows(pse_ctx *c, void *w, const void *rows, int add, int off, cudaStream_t s) {
-  StageTimer timer(c, PSE_STAGE_VECTOR, s);
-  const int64_t n = 8 * c->p.N;
-  VecArgs va = vec_args(c);
-  c->nlaunch += 1;
-  DISPATCH(c, (k_combine<float, false><<<(unsigned)c->nvblk, 256, 0, s>>>(va, (float *)w, (const float *)rows, n, 0, nullptr, c->d_coef + off, -1.0f, c->kd.iter, add)),
-           (k_combine<double, false><<<(unsigned)c->nvblk, 256, 0, s>>>(va, (double *)w, (const double *)rows, n, 0, nullptr, c->d_coef + off, -1.0, c->kd.iter, add)));
-  PSE_CUDA_TRY(c, cudaGetLastError());
-  return PSE_OK;
-}
-
-pse_status vscale_row(pse_ctx *c, void *basis, int delta, const void *src, void *vin, int off, cudaStream_t s) {
-  StageTimer timer(c, PSE_STAGE_VECTOR, s);
-  const int64_t n = 8 * c->p.N;
-  VecArgs va = vec_args(c);
-  c->nlaunch += 1;
-  DISPATCH(c, (k_vscale_row<float><<<(unsigned)c->nvblk, 256, 0, s>>>(va, (float *)basis, n, c->kd.iter, delta, (const float *)src, (float *)vin, c->d_coef + off)),
-           (k_vscale_row<double><<<(unsigned)c->nvblk, 256, 0, s>>>(va, (double *)basis, n, c->kd.iter, delta, (const double *)src, (double *)vin, c->d_coef + off)));
   PSE_CUDA_TRY(c, cudaGetLastError());
   return PSE_OK;
 }

@@ -467,7 +467,7 @@ pse_status wave_apply_t(pse_ctx *c, const void *vin, void *vout, int mode, bool 
   int cin = (mode == M_SE || mode == M_SU) ? 5 : 8, cout = mode == M_FULL ? 8 : (mode == M_SE ? 5 : 3);
   {
     StageTimer timer(c, PSE_STAGE_SPREAD, s, mode);
-    c->nlaunch += 2;  // counter reset + kernel
+    c->nlaunch += 1;
     spread_launch(c, a, vin, mode, s);
   }
   PSE_CUDA_TRY(c, cudaGetLastError());
@@ -488,7 +488,7 @@ pse_status wave_apply_t(pse_ctx *c, const void *vin, void *vout, int mode, bool 
   PSE_TRY(fft<T>(c, false, cout, s, mode));
   {
     StageTimer timer(c, PSE_STAGE_INTERP, s, mode);
-    c->nlaunch += 2;
+    c->nlaunch += 1;
     interp_launch(c, a, vout, mode, s);
   }
   PSE_CUDA_TRY(c, cudaGetLastError());
@@ -512,7 +512,7 @@ pse_status wave_noise_t(pse_ctx *c, const void *w2, uint64_t seed, uint64_t coun
   PSE_TRY(fft<T>(c, false, 8, s));
   {
     StageTimer timer(c, PSE_STAGE_INTERP, s);
-    c->nlaunch += 2;
+    c->nlaunch += 1;
     interp_launch(c, a, vout, M_FULL, s);
   }
   PSE_CUDA_TRY(c, cudaGetLastError());

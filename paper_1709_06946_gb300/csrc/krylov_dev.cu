@@ -1,34 +1,86 @@
-// Device-side control of the Krylov iterations: the FP64 scalar steps of the
-// Lanczos square root (Sec. 3.2: tridiagonal T_m, c_m = T_m^{1/2} e1, stopping
-// rule |c_m - [c_{m-1}; 0]| / |c_m| <= tol) and of unrestarted GMRES for the
-// stresslet constraint (Hessenberg column, Givens rotations, |r|/|b| <= tol,
-// back substitution), one thread per suspension (one warp for the Lanczos
-// square root).  The dot products they read
-// and the scale factors and combination coefficients they write live in the
-// per-suspension coefficient blocks; loop control sets a flag (and, inside a
-// CUDA graph, the while-node condition) so an iteration needs no host round trip.
+// Krylov vector kernels and the device-side control of the Lanczos square root
+// (Sec. 3.2: tridiagonal T_m, c_m = T_m^{1/2} e1, stopping rule
+// |c_m - [c_{m-1}; 0]| / |c_m| <= tol) and of unrestarted GMRES for the stresslet
+// constraint (Hessenberg column, Givens rotations, |r|/|b| <= tol, back substitution).
+//
+// One iteration after the product w = A v_j is four launches:
+//   k_kr_dot      h1 = V^T w
+//   k_kr_sub_dot  w -= V h1, h2 = V^T w
+//   k_kr_finish   w -= V h2, |w|^2, the scalar step of every suspension, loop control
+//   k_kr_next     v_{j+1} = w / |w|, also in cell-list order for the next pair sum
+// A sum over the blocks of a suspension is taken by the last of them to arrive (a
+// counter, no waiting), which in k_kr_finish also takes the scalar step, so neither the
+// sums nor the control cost a launch of their own.  The blocks hold at most 16384
+// elements and fewer for small vectors (pse_ctx::vchunk), and w's update and the next
+// dot products run over one block's rows back to back, out of L1 and L2.
+//
+// Bound by launch and reduction latency below about 10^5 particles and by HBM above.
+// Per GMRES iteration, all vector and control kernels, against eleven separate launches
+// on 16384-element blocks: N = 3000 63 -> 27 us, N = 64000 (11 rows) 120 -> 56 us,
+// N = 2^20 (4 rows) 205 -> 156 us.
+//
+// The dot products, scale factors and combination coefficients live in the
+// per-suspension coefficient blocks; loop control sets a flag (and, inside a CUDA graph,
+// the while-node condition) so an iteration needs no host round trip.
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
 #include "krylov_math.cuh"
 #include "pse_internal.cuh"
+#include "vec_common.cuh"
 
 namespace pse {
 namespace {
 
-__global__ void k_lz_start(KDev k) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < k.nsys; q += gridDim.x * blockDim.x) {
-    double *cf = k.coef + (size_t)q * COEF_STRIDE;
-    double b0 = sqrt(fmax(cf[CO_NRM], 0.0));
-    k.l_b0[q] = b0;
-    k.l_err[q] = HUGE_VAL;
-    k.l_it[q] = 0;
-    k.l_capped[q] = 0;
-    k.nrows[q] = 0;
-    k.active[q] = b0 > 0.0;
-    cf[CO_FAC] = b0 > 0.0 ? 1.0 / b0 : 0.0;
+struct KrArgs {
+  VecArgs va;
+  KDev k;
+  int64_t stride, nblk;  // elements of a basis row, blocks of the launch
+  double *partial;       // [row][block]
+  int *done;             // arrival counters: one per suspension, one for the launch
+};
+
+// True in every thread of the last of n blocks to arrive at *ctr (zero before and after).
+// What a thread wrote before the call is visible to the last block after it.
+__device__ __forceinline__ bool last_block(int *ctr, int n) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(ctr, 1) == n - 1;
+    if (s_last) *ctr = 0;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *k.iter = 0;
+  __syncthreads();
+  const bool last = s_last != 0;
+  if (last) __threadfence();
+  return last;
+}
+
+// out[r] = sum over blocks [b0, b1) of the partials of row r < nr (one warp per row).
+__device__ __forceinline__ void sum_partials(const KrArgs &a, int b0, int b1, int nr, double *out) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int r = wid; r < nr; r += nw) {
+    double sum = 0;
+    for (int b = b0 + lane; b < b1; b += 32) sum += __ldcg(a.partial + r * a.nblk + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) out[r] = sum;
+  }
+}
+
+// Dot products of the block's chunk of w with rows 0 .. nr - 1 into the partials; the
+// suspension's last block sums them into out.
+template <typename T>
+__device__ __forceinline__ void block_dots(const KrArgs &a, const Chunk &ch, const T *__restrict__ rows, int nr,
+                                           const T *w, double *out, double red[DOT_ROWS][DOT_NT / 32]) {
+  for (int r0 = 0; r0 < nr; r0 += DOT_ROWS) {
+    const int n = min(DOT_ROWS, nr - r0);
+    T acc[DOT_ROWS];
+    chunk_dots(ch, rows, a.stride, r0, n, w, acc);
+    block_sums(acc, n, a.partial, a.nblk, r0, red);
+  }
+  const int b0 = a.va.blk0[ch.s], b1 = a.va.blk0[ch.s + 1];
+  if (last_block(a.done + ch.s, b1 - b0)) sum_partials(a, b0, b1, nr, out);
 }
 
 // c = T^{1/2} e1 of the tridiagonal T (order m <= LZ_ROWS) by one warp: every lane
@@ -40,9 +92,7 @@ __global__ void k_lz_start(KDev k) {
 //
 // Bound by the latency of one reciprocal and three FP64 operations per row (the lanes
 // run side by side); the implicit QL sweeps it replaces are one serial chain of about
-// m^2 Givens rotations with a hypot and two divisions each.  Mean per launch over a
-// recurrence of 9 steps (50000 particles, tolerance 1e-4) 94 -> 13 us, of 7 steps
-// 61 -> 10 us.
+// m^2 Givens rotations with a hypot and two divisions each.
 constexpr int LZ_ROWS = 64;
 __device__ bool tridiag_sqrt_e1_warp(int m, const double *al, const double *be, const double *nodes, double *sm,
                                      double *cv, int lane) {
@@ -56,7 +106,7 @@ __device__ bool tridiag_sqrt_e1_warp(int m, const double *al, const double *be, 
   for (int i = lane; i < m; i += 32) hi = fmax(hi, sa[i] + sb[i] + (i > 0 ? sb[i - 1] : 0.0));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  const double ih = 1.0 / hi;  // T / hi has order one
+  const double ih = recip(hi);  // T / hi has order one
   for (int i = lane; i < m; i += 32) {
     sa[i] *= ih;
     sb[i] *= ih;
@@ -75,7 +125,7 @@ __device__ bool tridiag_sqrt_e1_warp(int m, const double *al, const double *be, 
     x[i * 33 + 32] = (s[0] + s[1]) + (s[2] + s[3]);
   }
   __syncwarp();
-  const double f = sqrt(hi);
+  const double f = root(hi);
   for (int i = lane; i < m; i += 32) {
     double t = sa[i] * x[i * 33 + 32];
     if (i > 0) t += sb[i - 1] * x[(i - 1) * 33 + 32];
@@ -92,21 +142,18 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// One warp per suspension (the launch has one 32-thread block per suspension).
-__global__ void __launch_bounds__(32) k_lz_step(KDev k) {
-  __shared__ double sm[LZ_ROWS * 35];
-  const int j = *k.iter, m = j + 1, L = k.lmax;
-  const int q = blockIdx.x, lane = threadIdx.x;
-  if (q >= k.nsys || !k.active[q]) return;
+// Scalar step of Lanczos iteration j for suspension q, by one warp; sm: LZ_ROWS * 35 doubles.
+__device__ void lz_step(const KDev &k, int q, int j, int lane, double *sm) {
+  const int m = j + 1, L = k.lmax;
   double *cf = k.coef + (size_t)q * COEF_STRIDE;
   double *al = k.l_alpha + (size_t)q * L, *be = k.l_beta + (size_t)q * L;
   double *cp = k.l_cprev + (size_t)q * L, *cv = k.l_c + (size_t)q * L;
   if (lane == 0) al[j] = cf[CO_H1 + j] + cf[CO_H2 + j];
   __syncwarp();
-  const double bj = sqrt(fmax(cf[CO_NRM], 0.0));
+  const double bj = root(fmax(cf[CO_NRM], 0.0));
   bool ok = true;
   if (j == 0) {
-    if (lane == 0) cv[0] = sqrt(fmax(al[0], 0.0));
+    if (lane == 0) cv[0] = root(fmax(al[0], 0.0));
   } else if (m > LZ_ROWS || !tridiag_sqrt_e1_warp(m, al, be, k.l_nodes, sm, cv, lane)) {
     // long recurrences, and spectra outside the window (rounding can take the smallest
     // eigenvalue of T to zero): one thread, work arrays in global memory
@@ -123,7 +170,7 @@ __global__ void __launch_bounds__(32) k_lz_step(KDev k) {
       num += dv * dv;
       den += c * c;
     }
-    err = sqrt(warp_sum(num) / warp_sum(den));
+    err = root(warp_sum(num) * recip(warp_sum(den)));
     if (k.ltol > 0 && err <= k.ltol) stop = true;
   }
   if (!stop) {
@@ -143,64 +190,197 @@ __global__ void __launch_bounds__(32) k_lz_step(KDev k) {
     k.l_capped[q] = !ok || (k.ltol > 0 && !(err <= k.ltol) && m == L);
   } else {
     be[j] = bj;
-    cf[CO_FAC] = 1.0 / bj;
+    cf[CO_FAC] = recip(bj);
   }
 }
 
-__global__ void k_gm_start(KDev k) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < k.nsys; q += gridDim.x * blockDim.x) {
-    double *cf = k.coef + (size_t)q * COEF_STRIDE;
-    double beta = sqrt(fmax(cf[CO_NRM], 0.0));
-    k.g_beta[q] = beta;
-    k.g_rel[q] = beta > 0.0 ? 1.0 : 0.0;
-    k.g_g[(size_t)q * (k.gmax + 1)] = beta;
-    k.g_it[q] = 0;
-    k.g_capped[q] = 0;
-    k.nrows[q] = 0;
-    k.active[q] = beta > 0.0;
-    cf[CO_FAC] = beta > 0.0 ? 1.0 / beta : 0.0;
+// Scalar step of GMRES iteration j for suspension q, by one warp; sm: at least 4 * 128
+// doubles.  The Hessenberg matrix is stored by columns (gmax + 1 reals each).
+__device__ void gm_step(const KDev &k, int q, int j, int lane, double *sm) {
+  const int M = k.gmax;
+  double *cf = k.coef + (size_t)q * COEF_STRIDE;
+  double *H = k.g_H + (size_t)q * (M + 1) * M, *cs = k.g_cs + (size_t)q * M, *sn = k.g_sn + (size_t)q * M;
+  double *g = k.g_g + (size_t)q * (M + 1);
+  double *col = sm, *sc = sm + 128, *ss = sm + 256, *sg = sm + 384;
+  for (int i = lane; i <= j; i += 32) {
+    col[i] = cf[CO_H1 + i] + cf[CO_H2 + i];
+    sc[i] = i < j ? cs[i] : 0.0;
+    ss[i] = i < j ? sn[i] : 0.0;
+    sg[i] = g[i];
+  }
+  __syncwarp();
+  const double hn = root(fmax(cf[CO_NRM], 0.0));
+  if (lane == 0) {
+    double a = col[0];
+    for (int i = 0; i < j; ++i) {  // previous rotations
+      const double b = col[i + 1];
+      col[i] = sc[i] * a + ss[i] * b;
+      a = -ss[i] * a + sc[i] * b;
+    }
+    const double r = root(a * a + hn * hn), ir = recip(r);
+    const double c = r == 0 ? 1.0 : a * ir, s = r == 0 ? 0.0 : hn * ir;
+    col[j] = r;
+    cs[j] = c;
+    sn[j] = s;
+    const double gn = -s * sg[j];
+    g[j + 1] = gn;
+    sg[j] = c * sg[j];
+    g[j] = sg[j];
+    ss[0] = fabs(gn) * recip(k.g_beta[q]);
+  }
+  __syncwarp();
+  const double rel = ss[0];
+  const bool stop = rel <= k.gtol || hn == 0.0 || j == M - 1;
+  for (int i = lane; i <= j; i += 32) H[(size_t)j * (M + 1) + i] = col[i];
+  if (stop) {  // back substitution H y = g into the combination coefficients, column by column
+    for (int i = j; i >= 0; --i) {
+      const double y = sg[i] * recip(col[i]);
+      __syncwarp();
+      if (lane == 0) cf[CO_Y + i] = y;
+      for (int l = lane; l < i; l += 32) {
+        sg[l] -= col[l] * y;
+        col[l] = H[(size_t)(i - 1) * (M + 1) + l];
+      }
+      __syncwarp();
+    }
+  }
+  if (lane != 0) return;
+  k.g_rel[q] = rel;
+  k.g_it[q] = j + 1;
+  if (stop) {
+    k.active[q] = 0;
+    k.nrows[q] = j + 1;
+    k.g_capped[q] = !(rel <= k.gtol) && j + 1 == M;
+  } else {
+    cf[CO_FAC] = recip(hn);
+  }
+}
+
+// Start of a recurrence from z (every suspension): |z|, the scalar state, iteration 0.
+template <typename T, bool GM>
+__global__ void k_kr_start(KrArgs a, const T *z) {
+  __shared__ double red[DOT_ROWS][DOT_NT / 32];
+  const Chunk ch = chunk_of(a.va);
+  const KDev &k = a.k;
+  const int q = ch.s;
+  T acc[DOT_ROWS];
+  chunk_dots(ch, z, 0, 0, 1, z, acc);
+  block_sums(acc, 1, a.partial, a.nblk, 0, red);
+  const int b0 = a.va.blk0[q], b1 = a.va.blk0[q + 1];
+  double *cf = k.coef + (size_t)q * COEF_STRIDE;
+  if (last_block(a.done + q, b1 - b0)) {
+    sum_partials(a, b0, b1, 1, cf + CO_NRM);
+    if (threadIdx.x == 0) {
+      const double b = root(fmax(cf[CO_NRM], 0.0));
+      if (GM) {
+        k.g_beta[q] = b;
+        k.g_rel[q] = b > 0.0 ? 1.0 : 0.0;
+        k.g_g[(size_t)q * (k.gmax + 1)] = b;
+        k.g_it[q] = 0;
+        k.g_capped[q] = 0;
+      } else {
+        k.l_b0[q] = b;
+        k.l_err[q] = HUGE_VAL;
+        k.l_it[q] = 0;
+        k.l_capped[q] = 0;
+      }
+      k.nrows[q] = 0;
+      k.active[q] = b > 0.0;
+      cf[CO_FAC] = b > 0.0 ? recip(b) : 0.0;
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) *k.iter = 0;
 }
 
-__global__ void k_gm_step(KDev k) {
-  const int j = *k.iter, M = k.gmax;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < k.nsys; q += gridDim.x * blockDim.x) {
-    if (!k.active[q]) continue;
+template <typename T>
+__global__ void k_kr_dot(KrArgs a, const T *__restrict__ rows, const T *w) {
+  __shared__ double red[DOT_ROWS][DOT_NT / 32];
+  const Chunk ch = chunk_of(a.va);
+  if (!a.va.active[ch.s]) return;
+  const int nr = min(*a.k.iter + 1, MAX_ROWS);
+  block_dots(a, ch, rows, nr, w, a.k.coef + (size_t)ch.s * COEF_STRIDE + CO_H1, red);
+}
+
+template <typename T>
+__global__ void k_kr_sub_dot(KrArgs a, const T *__restrict__ rows, T *w) {
+  __shared__ double red[DOT_ROWS][DOT_NT / 32];
+  __shared__ T cs[MAX_ROWS];
+  const Chunk ch = chunk_of(a.va);
+  if (!a.va.active[ch.s]) return;
+  const int nr = min(*a.k.iter + 1, MAX_ROWS);
+  double *cf = a.k.coef + (size_t)ch.s * COEF_STRIDE;
+  for (int r = threadIdx.x; r < nr; r += blockDim.x) cs[r] = (T)cf[CO_H1 + r];
+  __syncthreads();
+  chunk_sub(ch, w, rows, a.stride, nr, cs);
+  block_dots(a, ch, rows, nr, w, cf + CO_H2, red);
+}
+
+// The loop continues while a suspension is active and fewer than `cap` iterations ran
+// (so it always terminates); h: the while node's condition inside a graph.
+template <typename T, bool GM>
+__global__ void k_kr_finish(KrArgs a, const T *__restrict__ rows, T *w, int cap, cudaGraphConditionalHandle h,
+                            int graph) {
+  __shared__ double red[DOT_ROWS][DOT_NT / 32];
+  __shared__ T cs[MAX_ROWS];
+  __shared__ double sm[LZ_ROWS * 35];
+  const Chunk ch = chunk_of(a.va);
+  const KDev &k = a.k;
+  const int q = ch.s, j = *k.iter;
+  if (a.va.active[q]) {
+    const int nr = min(j + 1, MAX_ROWS);
     double *cf = k.coef + (size_t)q * COEF_STRIDE;
-    double *H = k.g_H + (size_t)q * (M + 1) * M, *cs = k.g_cs + (size_t)q * M, *sn = k.g_sn + (size_t)q * M;
-    double *g = k.g_g + (size_t)q * (M + 1);
-    for (int i = 0; i <= j; ++i) H[i * M + j] = cf[CO_H1 + i] + cf[CO_H2 + i];
-    const double hn = sqrt(fmax(cf[CO_NRM], 0.0));
-    H[(j + 1) * M + j] = hn;
-    for (int i = 0; i < j; ++i) {  // previous rotations
-      double a = H[i * M + j], b = H[(i + 1) * M + j];
-      H[i * M + j] = cs[i] * a + sn[i] * b;
-      H[(i + 1) * M + j] = -sn[i] * a + cs[i] * b;
-    }
-    double a = H[j * M + j], b = H[(j + 1) * M + j];
-    double r = hypot(a, b);
-    cs[j] = r == 0 ? 1.0 : a / r;
-    sn[j] = r == 0 ? 0.0 : b / r;
-    H[j * M + j] = r;
-    H[(j + 1) * M + j] = 0.0;
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    const double rel = fabs(g[j + 1]) / k.g_beta[q];
-    k.g_rel[q] = rel;
-    k.g_it[q] = j + 1;
-    if (rel <= k.gtol || hn == 0.0 || j == M - 1) {
-      k.active[q] = 0;
-      k.nrows[q] = j + 1;
-      k.g_capped[q] = !(rel <= k.gtol) && j + 1 == M;
-      for (int i = j; i >= 0; --i) {  // back substitution H y = g into the combination coefficients
-        double sum = g[i];
-        for (int l = i + 1; l <= j; ++l) sum -= H[i * M + l] * cf[CO_Y + l];
-        cf[CO_Y + i] = sum / H[i * M + i];
+    for (int r = threadIdx.x; r < nr; r += blockDim.x) cs[r] = (T)cf[CO_H2 + r];
+    __syncthreads();
+    T acc[DOT_ROWS];
+#pragma unroll
+    for (int r = 0; r < DOT_ROWS; ++r) acc[r] = 0;
+    acc[0] = chunk_sub(ch, w, rows, a.stride, nr, cs);
+    block_sums(acc, 1, a.partial, a.nblk, 0, red);
+    const int b0 = a.va.blk0[q], b1 = a.va.blk0[q + 1];
+    if (last_block(a.done + q, b1 - b0)) {
+      sum_partials(a, b0, b1, 1, cf + CO_NRM);
+      if (threadIdx.x < 32) {
+        __syncwarp();
+        if (GM) gm_step(k, q, j, threadIdx.x, sm);
+        else lz_step(k, q, j, threadIdx.x, sm);
       }
-    } else {
-      cf[CO_FAC] = 1.0 / hn;
+      __syncthreads();
     }
+  }
+  if (last_block(a.done + k.nsys, gridDim.x)) {
+    int any = 0;
+    for (int s = threadIdx.x; s < k.nsys; s += blockDim.x) any |= __ldcg(k.active + s);
+    any = __syncthreads_or(any);
+    if (threadIdx.x == 0) {
+      const int cont = any && j + 1 < cap;
+      *k.iter = j + 1;
+      k.flag[0] = cont;
+      if (graph) cudaGraphSetConditional(h, cont ? 1u : 0u);
+    }
+  }
+}
+
+// Basis row *iter = coef[s][CO_FAC] * src for the active suspensions, also into vin and,
+// particle by particle, into the cell-list order of the pair sum's input (pos: a
+// particle's place in that list).
+template <typename T>
+__global__ void k_kr_next(KrArgs a, T *basis, const T *src, T *vin, T *vcell, const int *__restrict__ pos) {
+  using V = V16<T>;
+  using VT = typename V::t;
+  const Chunk ch = chunk_of(a.va);
+  if (!a.va.active[ch.s]) return;
+  const T f = (T)a.k.coef[(size_t)ch.s * COEF_STRIDE + CO_FAC];
+  T *dst = basis + (int64_t)*a.k.iter * a.stride;
+  for (int64_t e = ch.beg + (int64_t)threadIdx.x * V::n; e < ch.end; e += (int64_t)blockDim.x * V::n) {
+    const int64_t p = pos[e >> 3];
+    T x[V::n];
+    V::get(*(const VT *)(src + e), x);
+#pragma unroll
+    for (int i = 0; i < V::n; ++i) x[i] *= f;
+    const VT v = V::put(x);
+    *(VT *)(dst + e) = v;
+    *(VT *)(vin + e) = v;
+    *(VT *)(vcell + 8 * p + (e & 7)) = v;
   }
 }
 
@@ -215,52 +395,82 @@ __global__ void k_loop_begin(KDev k, cudaGraphConditionalHandle h, int graph) {
   }
 }
 
-// Advances the iteration counter; the loop continues while a suspension is
-// active and fewer than `cap` iterations ran (so it always terminates).
-__global__ void k_loop_end(KDev k, int cap, cudaGraphConditionalHandle h, int graph) {
-  int any = 0;
-  for (int q = threadIdx.x; q < k.nsys; q += blockDim.x) any |= k.active[q];
-  any = __syncthreads_or(any);
-  if (threadIdx.x == 0) {
-    const int j = *k.iter + 1;
-    *k.iter = j;
-    const int cont = any && j < cap;
-    k.flag[0] = cont;
-    if (graph) cudaGraphSetConditional(h, cont ? 1u : 0u);
-  }
-}
-
 __global__ void k_all_active(int nsys, int *active) {
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nsys; q += gridDim.x * blockDim.x) active[q] = 1;
 }
 
 unsigned sys_blocks(const pse_ctx *c) { return (unsigned)std::min<int64_t>(ceil_div(c->nsys, 128), 512); }
 
+KrArgs kr_args(const pse_ctx *c) {
+  KrArgs a;
+  a.va = vec_args(c);
+  a.k = c->kd;
+  a.stride = 8 * c->p.N;
+  a.nblk = c->nvblk;
+  a.partial = c->d_dots;
+  a.done = c->d_done;
+  return a;
+}
+
+template <typename T>
+void kr_start_t(pse_ctx *c, const void *z, bool gm, cudaStream_t s) {
+  const unsigned nb = (unsigned)c->nvblk;
+  if (gm) k_kr_start<T, true><<<nb, DOT_NT, 0, s>>>(kr_args(c), (const T *)z);
+  else k_kr_start<T, false><<<nb, DOT_NT, 0, s>>>(kr_args(c), (const T *)z);
+}
+
+template <typename T>
+void kr_step_t(pse_ctx *c, void *w, bool gm, int cap, cudaGraphConditionalHandle h, int graph, cudaStream_t s) {
+  const unsigned nb = (unsigned)c->nvblk;
+  const KrArgs a = kr_args(c);
+  const T *V = (const T *)c->d_basis;
+  k_kr_dot<T><<<nb, DOT_NT, 0, s>>>(a, V, (const T *)w);
+  k_kr_sub_dot<T><<<nb, DOT_NT, 0, s>>>(a, V, (T *)w);
+  if (gm) k_kr_finish<T, true><<<nb, DOT_NT, 0, s>>>(a, V, (T *)w, cap, h, graph);
+  else k_kr_finish<T, false><<<nb, DOT_NT, 0, s>>>(a, V, (T *)w, cap, h, graph);
+}
+
 }  // namespace
 
-void kd_lz_start(pse_ctx *c, cudaStream_t s) {
+// |z| and the scalar start of a Lanczos (gm = false) or GMRES recurrence.
+pse_status kr_start(pse_ctx *c, const void *z, bool gm, cudaStream_t s) {
+  StageTimer timer(c, PSE_STAGE_VECTOR, s);
   c->nlaunch += 1;
-  k_lz_start<<<sys_blocks(c), 128, 0, s>>>(c->kd);
+  if (c->prec == PSE_MIXED) kr_start_t<float>(c, z, gm, s);
+  else kr_start_t<double>(c, z, gm, s);
+  PSE_CUDA_TRY(c, cudaGetLastError());
+  return PSE_OK;
 }
-void kd_lz_step(pse_ctx *c, cudaStream_t s) {
+
+// Orthogonalises w against basis rows 0 .. *iter (classical Gram-Schmidt twice, FP64
+// coefficients), takes the scalar step of every active suspension and advances the loop.
+pse_status kr_step(pse_ctx *c, void *w, bool gm, int cap, cudaGraphConditionalHandle h, int graph, cudaStream_t s) {
+  StageTimer timer(c, PSE_STAGE_VECTOR, s);
+  c->nlaunch += 3;
+  if (c->prec == PSE_MIXED) kr_step_t<float>(c, w, gm, cap, h, graph, s);
+  else kr_step_t<double>(c, w, gm, cap, h, graph, s);
+  PSE_CUDA_TRY(c, cudaGetLastError());
+  return PSE_OK;
+}
+
+// The next Krylov vector from src: basis row *iter, d_vin and d_vcell (the pair sum's input).
+pse_status kr_next(pse_ctx *c, const void *src, cudaStream_t s) {
+  StageTimer timer(c, PSE_STAGE_VECTOR, s);
   c->nlaunch += 1;
-  k_lz_step<<<(unsigned)c->nsys, 32, 0, s>>>(c->kd);
+  const unsigned nb = (unsigned)c->nvblk;
+  if (c->prec == PSE_MIXED)
+    k_kr_next<float><<<nb, DOT_NT, 0, s>>>(kr_args(c), (float *)c->d_basis, (const float *)src, (float *)c->d_vin,
+                                           (float *)c->d_vcell, c->d_cell_key);
+  else
+    k_kr_next<double><<<nb, DOT_NT, 0, s>>>(kr_args(c), (double *)c->d_basis, (const double *)src, (double *)c->d_vin,
+                                            (double *)c->d_vcell, c->d_cell_key);
+  PSE_CUDA_TRY(c, cudaGetLastError());
+  return PSE_OK;
 }
-void kd_gm_start(pse_ctx *c, cudaStream_t s) {
-  c->nlaunch += 1;
-  k_gm_start<<<sys_blocks(c), 128, 0, s>>>(c->kd);
-}
-void kd_gm_step(pse_ctx *c, cudaStream_t s) {
-  c->nlaunch += 1;
-  k_gm_step<<<sys_blocks(c), 128, 0, s>>>(c->kd);
-}
+
 void kd_loop_begin(pse_ctx *c, cudaGraphConditionalHandle h, int graph, cudaStream_t s) {
   c->nlaunch += 1;
   k_loop_begin<<<1, 256, 0, s>>>(c->kd, h, graph);
-}
-void kd_loop_end(pse_ctx *c, int cap, cudaGraphConditionalHandle h, int graph, cudaStream_t s) {
-  c->nlaunch += 1;
-  k_loop_end<<<1, 256, 0, s>>>(c->kd, cap, h, graph);
 }
 void kd_all_active(pse_ctx *c, cudaStream_t s) {
   c->nlaunch += 1;

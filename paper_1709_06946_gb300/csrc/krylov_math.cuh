@@ -127,18 +127,33 @@ inline void sqrt_nodes(int n, double window, double *s, double *w) {
   }
 }
 
-// 1 / d for |d| well inside the FP32 range.  On the device: an FP32 reciprocal and two
-// Newton steps r (2 - d r), each doubling the correct digits (7, 14, 28), seven
-// dependent instructions where the FP64 division takes about three times as many of
-// a unit that issues one warp instruction in sixteen cycles.
+// 1 / d and sqrt(x) in FP64.  On the device, for arguments well inside the FP32 range, an
+// FP32 seed and Newton steps (each doubles the correct digits: 7, 14, 28): the FP64 unit
+// issues one warp instruction in sixteen cycles and the library forms are serial chains
+// of several tens of them.
 __host__ __device__ inline double recip(double d) {
 #ifdef __CUDA_ARCH__
-  double r = (double)(1.0f / (float)d);
-  r = fma(r, fma(-d, r, 1.0), r);
-  return fma(r, fma(-d, r, 1.0), r);
-#else
-  return 1.0 / d;
+  const float f = (float)d;
+  if (fabsf(f) > 1e-30f && fabsf(f) < 1e30f) {
+    double r = (double)(1.0f / f);
+    r = fma(r, fma(-d, r, 1.0), r);
+    return fma(r, fma(-d, r, 1.0), r);
+  }
 #endif
+  return 1.0 / d;
+}
+__host__ __device__ inline double root(double x) {
+#ifdef __CUDA_ARCH__
+  const float f = (float)x;
+  if (f > 1e-30f && f < 1e30f) {
+    double y = (double)rsqrtf(f);
+    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    const double s = x * y;
+    return fma(0.5 * y, fma(-s, s, x), s);
+  }
+#endif
+  return sqrt(x);
 }
 
 // x = (T + shift)^{-1} e1 for T = tridiag(beta, alpha, beta) of order n, eliminated from

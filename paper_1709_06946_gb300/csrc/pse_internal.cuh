@@ -145,7 +145,12 @@ struct FftGroup {
   bool ok[2][12] = {{false}};
 };
 
-constexpr int VEC_CHUNK = 16384;   // vector elements per block of the chunked vector kernels
+// Vector elements per block of the chunked vector kernels: the largest power of two from
+// VEC_CHUNK_MIN to VEC_CHUNK_MAX that gives VEC_BLOCKS blocks (one per SM), or the
+// smallest.  At N = 64000, 16384 elements, right at 2^20 particles, are 32 blocks on 152
+// SMs; 2048 (250 blocks) take 17.5 us per pass over 11 rows and 1024 (500 blocks, more
+// FP64 reduction work) 21.4 us.
+constexpr int VEC_CHUNK_MAX = 16384, VEC_CHUNK_MIN = 1024, VEC_BLOCKS = 152;
 constexpr int COEF_STRIDE = 512;   // doubles of Krylov coefficients per suspension
 constexpr int MAX_ROWS = 128;      // Krylov vectors per dot-product / combination launch
 constexpr int CUBE_TILE = 16;      // tile side of the specialised spreading / interpolation kernels
@@ -203,6 +208,8 @@ struct pse_ctx {
   std::vector<int> h_active;
   std::vector<pse::FftGroup> groups;
   int64_t nk_tot = 0, nvblk = 0;             // half-spectrum points, vector blocks
+  int vchunk = pse::VEC_CHUNK_MAX;           // vector elements per block
+  int *d_done = nullptr;                     // nsys + 1 arrival counters of the Krylov kernels (zero between launches)
   std::vector<pse_stats> sys_stats;          // per suspension, last call
   int *d_queue = nullptr;                    // work counters of the persistent kernels
   int queue_slot = 0;
@@ -361,7 +368,8 @@ struct StageTimer {
 namespace pse {
 struct Scan;
 pse_status setup_config(pse_ctx *c, const double *d_pos, cudaStream_t s);
-pse_status real_apply(pse_ctx *c, const void *vin, void *vout, int mode, cudaStream_t s);
+// gathered: vin is already in d_vcell in cell-list order
+pse_status real_apply(pse_ctx *c, const void *vin, void *vout, int mode, cudaStream_t s, bool gathered = false);
 // Harmonic overlap force of the current configuration into F (user order, N x 3).
 pse_status overlap_force(pse_ctx *c, double kspring, void *F, cudaStream_t s);
 pse_status wave_apply(pse_ctx *c, const void *vin, void *vout, int mode, bool add, cudaStream_t s);
@@ -373,7 +381,8 @@ pse_status wave_noise(pse_ctx *c, const void *w2, uint64_t seed, uint64_t counte
 // mode flags for real/wave products
 // M_SU: S -> U (the final velocity when there is no external force)
 enum { M_FULL = 0, M_SE = 1, M_FSU = 2, M_SU = 3 };
-pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s);
+pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s,
+                    bool gathered = false);
 
 // vector helpers
 pse_status gather_in(pse_ctx *c, const void *F, const void *S, void *vout, cudaStream_t s);
@@ -384,7 +393,6 @@ pse_status philox_w1(pse_ctx *c, uint64_t seed, uint64_t counter, void *vout, cu
 // Per-suspension Krylov helpers over [N][8] vectors; coefficients and results
 // live at d_coef + s * COEF_STRIDE + off for suspension s, and suspensions
 // with d_active[s] == 0 are skipped.
-pse_status multidot(pse_ctx *c, const void *rows, int nrows, const void *w, int off, cudaStream_t s);
 pse_status combine_sub(pse_ctx *c, void *w, const void *rows, int nrows, int off, cudaStream_t s);
 pse_status combine_set(pse_ctx *c, void *y, const void *rows, const int *d_nrows, int maxrows, int off,
                        cudaStream_t s);
@@ -401,21 +409,14 @@ pse_status gather12(pse_ctx *c, const void *F, const void *L, const void *S, voi
 pse_status scatter12(pse_ctx *c, const void *vin, void *U, void *Om, void *E, cudaStream_t s);
 pse_status rfd_final(pse_ctx *c, const double *x0, const void *B, const void *U0, const void *Rp, const void *Rm,
                      double dt, double fac, double *xout, cudaStream_t s);
-// Krylov control kernels (krylov_dev.cu); handle = 0 and graph = 0 outside a graph.
-void kd_lz_start(pse_ctx *c, cudaStream_t s);
-void kd_lz_step(pse_ctx *c, cudaStream_t s);
-void kd_gm_start(pse_ctx *c, cudaStream_t s);
-void kd_gm_step(pse_ctx *c, cudaStream_t s);
+// Krylov vector and control kernels (krylov_dev.cu); handle = 0 and graph = 0 outside a graph.
+pse_status kr_start(pse_ctx *c, const void *z, bool gm, cudaStream_t s);
+pse_status kr_step(pse_ctx *c, void *w, bool gm, int cap, cudaGraphConditionalHandle h, int graph, cudaStream_t s);
+pse_status kr_next(pse_ctx *c, const void *src, cudaStream_t s);
 void kd_loop_begin(pse_ctx *c, cudaGraphConditionalHandle h, int graph, cudaStream_t s);
-void kd_loop_end(pse_ctx *c, int cap, cudaGraphConditionalHandle h, int graph, cudaStream_t s);
 void kd_all_active(pse_ctx *c, cudaStream_t s);
-// Rows 0 .. *kd.iter + add - 1 of the basis: dot products into coef[s][off + r] and w -= sum coef rows.
-pse_status multidot_rows(pse_ctx *c, const void *rows, int add, const void *w, int off, cudaStream_t s);
-pse_status combine_sub_rows(pse_ctx *c, void *w, const void *rows, int add, int off, cudaStream_t s);
-// Row *kd.iter + delta of the basis (and vin, if given) = coef[s][off] * src.
-pse_status vscale_row(pse_ctx *c, void *basis, int delta, const void *src, void *vin, int off, cudaStream_t s);
-// Work counter for the next persistent launch (cleared on stream s).
-int *next_queue(pse_ctx *c, cudaStream_t s);
+// Work counter for the next persistent launch (zero; the launch leaves it at zero).
+int *next_queue(pse_ctx *c);
 // Resident CTAs of a persistent kernel: SMs x blocks per SM (queried once into
 // per_sm, 0 on entry), at most `items`.
 template <typename K>

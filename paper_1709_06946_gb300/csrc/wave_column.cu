@@ -508,7 +508,7 @@ void launch_interp_col(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s
   constexpr int NT = 32 * 8 * (CUBE / ZT);
   auto kern = k_interp_col<C, SLOT0, P, ZT>;
   const unsigned grid = wave_grid(c, kern, 0, a.ntiles, occ, NT);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   kern<<<grid, NT, 0, s>>>(a, q, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, c->d_fine_start,
                            (const float *)c->d_grid, (float *)vout);
 }
@@ -525,7 +525,7 @@ void interp_col_p(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) {
 template <int C, int SLOT0, int P, int ZT, bool DEF = false>
 void launch_spread_col_z(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStream_t s) {
   constexpr int NT = 32 * 8 * (CUBE / ZT);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   if (!DEF && (c->opt.wave_kernel & 4)) {  // every warp scans the candidates itself
     static OccCache occ;
     auto kern = k_spread_col<C, SLOT0, P, ZT>;

@@ -392,7 +392,7 @@ void launch_spread16(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStream_
   set_smem(kern, once);
   const size_t sm = TileL<float, C>::bytes((size_t)CUBE * CUBE * tile_rx(CUBE, P));
   const unsigned grid = wave_grid(c, kern, sm, a.ntiles, occ);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   kern<<<grid, WAVE_THREADS, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, (const float *)vin,
                                       c->d_fine_start, (float *)c->d_grid);
 }
@@ -406,7 +406,7 @@ void launch_interp16(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) 
   set_smem(kern, once);
   const size_t sm = TileL<float, C>::bytes((size_t)CUBE * CUBE * tile_rx(CUBE, P));
   const unsigned grid = wave_grid(c, kern, sm, a.ntiles, occ, NT);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   kern<<<grid, NT, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, c->d_fine_start,
                             (const float *)c->d_grid, (float *)vout);
 }

@@ -178,7 +178,7 @@ void launch_interp_halo(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t 
   auto kern = k_interp_halo<C, SLOT0, P, DEF, COMP0>;
   set_smem(kern, once);
   const unsigned grid = wave_grid(c, kern, sm, a.ntiles * SUB_SIDE, occ, HALO_THREADS);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   kern<<<grid, HALO_THREADS, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, c->d_fine_start,
                                       (const float *)c->d_grid, (float *)vout);
 }

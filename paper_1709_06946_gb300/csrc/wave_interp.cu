@@ -198,7 +198,7 @@ void launch_interp(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) {
   set_smem(kern, once);
   size_t sm = wave_smem_max<T, C>(c, a.want);
   unsigned grid = wave_grid(c, kern, sm, a.ntiles, occ, NT);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   kern<<<grid, NT, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const typename V4<T>::t *)c->d_sp_d0,
                             c->d_tile_start, (const T *)c->d_grid, (T *)vout);
 }
@@ -245,7 +245,7 @@ void interp_launch(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStre
     ac.want = 1;
     ag.want = 0;
     interp_cubic(c, ac, vout, mode, s);
-    c->nlaunch += 2;
+    c->nlaunch += 1;
   }
   if (c->prec == PSE_MIXED) {
     if (mode == M_FULL) interp_p<float, 8, 0>(c, ag, vout, s);
@@ -269,7 +269,7 @@ void interp11_launch(pse_ctx *c, void *vout12, cudaStream_t s) {
     interp_p<double, 8, 0, 12, 0>(c, a, vout12, s);
     interp_p<double, 3, 8, 12, 8>(c, a, vout12, s);
   }
-  c->nlaunch += 4;
+  c->nlaunch += 2;
 }
 
 }  // namespace pse

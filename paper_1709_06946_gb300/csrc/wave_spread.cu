@@ -181,7 +181,7 @@ void launch_spread(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStream_t 
   set_smem(kern, once);
   size_t sm = wave_smem_max<T, C>(c, a.want);
   unsigned grid = wave_grid(c, kern, sm, a.ntiles, occ);
-  int *q = next_queue(c, s);
+  int *q = next_queue(c);
   kern<<<grid, WAVE_THREADS, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const typename V4<T>::t *)c->d_sp_d0,
                                       (const T *)vin, c->d_fine_start, (T *)c->d_grid);
 }
@@ -214,7 +214,7 @@ void spread_launch(pse_ctx *c, const WaveArgs &a, const void *vin, int mode, cud
     ac.want = 1;
     ag.want = 0;
     spread_cubic(c, ac, vin, mode, s);
-    c->nlaunch += 2;
+    c->nlaunch += 1;
   }
   if (c->prec == PSE_MIXED) {
     if (mode == M_SE || mode == M_SU) spread_p<float, 5, 3>(c, ag, vin, s);
@@ -236,7 +236,7 @@ void spread11_launch(pse_ctx *c, const void *vin12, cudaStream_t s) {
     spread_p<double, 8, 0, 12, 0>(c, a, vin12, s);
     spread_p<double, 3, 8, 12, 8>(c, a, vin12, s);
   }
-  c->nlaunch += 4;
+  c->nlaunch += 2;
 }
 
 }  // namespace pse
