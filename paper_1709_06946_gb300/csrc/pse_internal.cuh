@@ -245,7 +245,7 @@ struct pse_ctx {
   unsigned long long *h_nbr_tot = nullptr;  // pinned copy
   void *d_sp_i0 = nullptr;      // int4 per particle: wrapped support start
   void *d_sp_d0 = nullptr;      // real4: i0*h - x per dimension
-  void *d_rs = nullptr;         // float4 (cell offset + packed cell) or double4_32a positions
+  void *d_rs = nullptr;         // float4 (cell offset, x cell index) or double4_32a positions
   int *d_scan_tmp = nullptr;    // block sums for scans
   int64_t ntiles = 0, ncells = 0;
   int64_t tile_cap = 0, scan_cap = 0;  // allocated tile-array and scan-scratch capacities
