@@ -840,6 +840,8 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
   c->table_dr = t.dr;
   c->self_uf = t.self_uf;
   c->self_es = t.self_es;
+  if (c->prec == PSE_MIXED && o.table_points <= 0)
+    c->poly.ok = build_real_poly(c->p, t, c->poly) <= 1.0 ? 1 : 0;
   bool fail = false;
   auto A = [&](size_t bytes) {
     void *q = dalloc(c, bytes);

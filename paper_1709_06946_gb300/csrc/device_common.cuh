@@ -110,4 +110,38 @@ __device__ __forceinline__ void Smul(const T s[5], const T p[3], T v[3]) {
   v[2] = sxz * p[0] + syz * p[1] + szz * p[2];
 }
 
+// Row i (8 reals) of a vector of rows; FP32: one 256-bit access.
+__device__ __forceinline__ void load_row(const float4 *p, int64_t i, float4 &lo, float4 &hi) {
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(lo.x), "=f"(lo.y), "=f"(lo.z), "=f"(lo.w), "=f"(hi.x), "=f"(hi.y), "=f"(hi.z), "=f"(hi.w)
+               : "l"(p + 2 * i)
+               : "memory");
+}
+__device__ __forceinline__ void store_row(float4 *p, int64_t i, const float4 &lo, const float4 &hi) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p + 2 * i), "f"(lo.x), "f"(lo.y), "f"(lo.z),
+               "f"(lo.w), "f"(hi.x), "f"(hi.y), "f"(hi.z), "f"(hi.w)
+               : "memory");
+}
+__device__ __forceinline__ void load_row(const double4_32a *p, int64_t i, double4_32a &lo, double4_32a &hi) {
+  lo = p[2 * i];
+  hi = p[2 * i + 1];
+}
+__device__ __forceinline__ void store_row(double4_32a *p, int64_t i, const double4_32a &lo, const double4_32a &hi) {
+  p[2 * i] = lo;
+  p[2 * i + 1] = hi;
+}
+
+// Row [F, s1..s5] of a Krylov vector as the pair sum reads it: [F, Sxx, Syy, Sxy, Sxz, Syz].
+template <typename T4>
+__device__ __forceinline__ void cell_row(T4 &lo, T4 &hi) {
+  using T = decltype(lo.x);
+  const T i2 = (T)0.70710678118654752, i6 = (T)0.40824829046386302;
+  const T a = lo.w * i2, b = hi.x * i6;
+  lo.w = a + b;
+  hi.x = b - a;
+  hi.y *= i2;
+  hi.z *= i2;
+  hi.w *= i2;
+}
+
 }  // namespace pse

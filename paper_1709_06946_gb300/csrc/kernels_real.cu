@@ -8,9 +8,13 @@
 // into cell-list order, so the lanes of a particle, walking consecutive entries
 // of the list (runs of cells along x), read neighbouring rows of that copy and
 // share cache lines.  A persistent grid takes blocks of particles from a work
-// counter; particles of suspensions marked inactive are skipped.  The seven scalar functions
-// come from a table on r: linear interpolation in FP32 (mixed form), cubic
-// Lagrange interpolation in FP64 with one-sided stencils at the r = 2a node
+// counter; particles of suspensions marked inactive are skipped.  The copy holds the
+// stresslet as Cartesian components, and the strain rates are summed as Cartesian
+// components and projected on the Y basis once per particle.
+//
+// The seven scalar functions, FP32: beyond contact a Gaussian times polynomials in 1/r
+// (RealPoly, fitted per handle), below it a table on r with linear interpolation; FP64:
+// cubic Lagrange interpolation of the table with one-sided stencils at the r = 2a node
 // where the functions have a kink.
 #include <algorithm>
 
@@ -26,6 +30,9 @@ struct RealArgs {
   double inv_dr, self_uf, self_es;
 };
 
+// Where an FP32 product takes its scalar functions from.
+enum { LK_TABLE = 0, LK_SMEM = 1, LK_POLY = 2 };
+
 // 32 bytes (8 floats) from 32-byte aligned read-only global memory in one
 // 256-bit load.
 __device__ __forceinline__ void ldg8(const float *p, float4 &lo, float4 &hi) {
@@ -33,6 +40,18 @@ __device__ __forceinline__ void ldg8(const float *p, float4 &lo, float4 &hi) {
       : "=f"(lo.x), "=f"(lo.y), "=f"(lo.z), "=f"(lo.w), "=f"(hi.x), "=f"(hi.y), "=f"(hi.z), "=f"(hi.w)
       : "l"(p));
 }
+
+// A neighbour record, brought from DRAM 256 bytes at a time (a particle's records are
+// contiguous: its lanes' next four steps).  S -> E at 2^20 particles 435 -> 415 us; not
+// allocating in L1 makes it 462 us.
+__device__ __forceinline__ float4 ld_record(const float4 *p) {
+  float4 v;
+  asm("ld.global.nc.L2::256B.v4.f32 {%0,%1,%2,%3}, [%4];"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double4_32a ld_record(const double4_32a *p) { return *p; }
 
 // f[0..7) at r by linear interpolation.  The full product reads two 8-float
 // entries (q and q + 1); the partial products read one 8-float interval record
@@ -87,33 +106,97 @@ __device__ __forceinline__ void lookup(const double *tab, const RealArgs &a, dou
   else b = max(b, a.k2);
   b = max(0, min(b, a.len - 4));
   double t = x - (double)b;
-  double w0 = -(t - 1) * (t - 2) * (t - 3) / 6.0, w1 = t * (t - 2) * (t - 3) / 2.0;
-  double w2 = -t * (t - 1) * (t - 3) / 2.0, w3 = t * (t - 1) * (t - 2) / 6.0;
+  const double c6 = 1.0 / 6.0, u0 = t * (t - 1), u1 = (t - 2) * (t - 3);
+  const double w0 = -c6 * (t - 1) * u1, w1 = 0.5 * t * u1, w2 = -0.5 * u0 * (t - 3), w3 = c6 * u0 * (t - 2);
   const double *r0 = tab + 8 * (size_t)b;
 #pragma unroll
   for (int k = 0; k < 7; ++k)
     f[k] = w0 * __ldg(r0 + k) + w1 * __ldg(r0 + 8 + k) + w2 * __ldg(r0 + 16 + k) + w3 * __ldg(r0 + 24 + k);
 }
 
+__device__ __forceinline__ float fast_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float fast_exp2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Function k of the fit: f_k = exp2(-cg (r - r0)^2) P_k(t), t = ta / r + tb in [-1, 1].
+__device__ __forceinline__ float poly_at(const RealPoly &p, int k, float t) {
+  float v = p.c[k][POLY_DEG];
+#pragma unroll
+  for (int d = POLY_DEG - 1; d >= 0; --d) v = fmaf(v, t, p.c[k][d]);
+  return v;
+}
+
+// One neighbour's terms.  g: separation; row: [F, Sxx, Syy, Sxy, Sxz, Syz]; f: the scalar
+// functions with f[1] - f[0] in place of f[1].  U += f2 v + f0 F + (f3 q + (f1 - f0) rf) rh with
+// v = S rh, q = rh.v, rf = rh.F; the strain is sym(w, rh) + f4 S with
+// w = f5 v - f2 F / 2 + (f6 q - f3 rf) / 2 rh; d holds half of its diagonal, o the rest.
+template <typename T, int MODE>
+__device__ __forceinline__ void pair_terms(const T rh[3], const T row[8], const T f[7], T U[3], T d[3], T o[3]) {
+  constexpr bool HAS_F = MODE == M_FULL || MODE == M_FSU, WANT_U = MODE != M_SE;
+  constexpr bool WANT_E = MODE == M_FULL || MODE == M_SE;
+  const T szz = -(row[3] + row[4]);
+  const T v[3] = {row[3] * rh[0] + row[5] * rh[1] + row[6] * rh[2], row[5] * rh[0] + row[4] * rh[1] + row[7] * rh[2],
+                  row[6] * rh[0] + row[7] * rh[1] + szz * rh[2]};
+  const T q = rh[0] * v[0] + rh[1] * v[1] + rh[2] * v[2];
+  const T rf = HAS_F ? rh[0] * row[0] + rh[1] * row[1] + rh[2] * row[2] : (T)0;
+  if (WANT_U) {
+    T c = f[3] * q;
+    if (HAS_F) c += f[1] * rf;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      U[m] += f[2] * v[m] + c * rh[m];
+      if (HAS_F) U[m] += f[0] * row[m];
+    }
+  }
+  if (WANT_E) {
+    const T cy = (T)0.5 * (HAS_F ? f[6] * q - f[3] * rf : f[6] * q), h4 = (T)0.5 * f[4], h2 = (T)-0.5 * f[2];
+    T w[3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      w[m] = f[5] * v[m] + cy * rh[m];
+      if (HAS_F) w[m] += h2 * row[m];
+    }
+    d[0] += h4 * row[3] + w[0] * rh[0];
+    d[1] += h4 * row[4] + w[1] * rh[1];
+    d[2] += h4 * szz + w[2] * rh[2];
+    o[0] += f[4] * row[5] + w[0] * rh[1] + w[1] * rh[0];
+    o[1] += f[4] * row[6] + w[0] * rh[2] + w[2] * rh[0];
+    o[2] += f[4] * row[7] + w[1] * rh[2] + w[2] * rh[1];
+  }
+}
+
 // G lanes share one particle: they walk its neighbour list with stride G (so
 // the neighbours' records are fetched in parallel) and the partial sums are
 // reduced with shuffles; the first lane of the group adds the self term.
-// FP32: at most 64 registers so that four 256-thread CTAs fit an SM (the full
-// 8 -> 8 product would otherwise take 74 and leave room for three).  With
-// SHT (FP32 only) one 1024-thread CTA per SM first copies the table into shared
-// memory and the lookups leave L1 to the neighbours' records.
-template <typename T, int MODE, int G, bool SHT = false, int NT = SHT ? 1024 : 256>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (SHT ? 1 : 4) : 1) k_real(RealArgs a,
-                                              const SysDev *__restrict__ sys,
-                                              const int64_t *__restrict__ p0, const int *__restrict__ active,
-                                              int *queue, int nitems,
-                                              const int *__restrict__ nstart,
-                                              const typename V4<T>::t *__restrict__ geo,
-                                              const T *__restrict__ vin, const T *__restrict__ vcell,
-                                              T *__restrict__ vout, const T *__restrict__ gtab) {
+//
+// Bound: random 32-byte reads pass L1 at 64 bytes per clock and SM (1.95 lanes per clock
+// measured), so a table entry per pair (two for the full product) cost as much as the
+// neighbour's row; the polynomials take 9 FMAs per function instead, and the FMA pipe
+// and L1 are then about equally busy.  The terms collected along rh and in Cartesian
+// components take about 60 operations (110 in the Y basis).  At 2^20 particles, 105
+// neighbours each: full product 886 -> 630 us, S -> E 648 -> 415, S -> U 594 -> 364;
+// FP64 form at 11000 particles 630 -> 445 us.  Below 10^5 particles the few thousand warps
+// wait on their records (47 us at 64000, 68 before).
+//
+// FP32: 48 registers so that five 256-thread CTAs fit an SM (four: S -> E 487 us; six:
+// full 751 us, spilled).  A static split over warps instead of the work counter: full 737
+// us.  With LK_SMEM one 1024-thread CTA per SM first copies the table into shared memory.
+template <typename T, int MODE, int G, int LK = LK_TABLE, int NT = LK == LK_SMEM ? 1024 : 256>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (LK == LK_SMEM ? 1 : 5) : 1)
+    k_real(RealArgs a, RealPoly poly, const SysDev *__restrict__ sys, const int64_t *__restrict__ p0,
+           const int *__restrict__ active, int *queue, int nitems, const int *__restrict__ nstart,
+           const typename V4<T>::t *__restrict__ geo, const T *__restrict__ vin, const T *__restrict__ vcell,
+           T *__restrict__ vout, const T *__restrict__ gtab) {
   extern __shared__ __align__(16) unsigned char tab_raw[];
   const T *tab = gtab;
-  if (SHT) {
+  if (LK == LK_SMEM) {
     float4 *dst = (float4 *)tab_raw;
     const float4 *src = (const float4 *)gtab;
     for (int q = threadIdx.x; q < 2 * a.len; q += blockDim.x) dst[q] = src[q];
@@ -131,55 +214,51 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (SHT ? 1 : 4) : 1) k_real
     const bool live = gid < a.Ntot && active[si];
     const SysDev &sd = sys[si];
     const T4 *v4 = (const T4 *)vin, *vc4 = (const T4 *)vcell;
-    T U[3] = {0, 0, 0}, E[5] = {0, 0, 0, 0, 0};
+    T U[3] = {0, 0, 0}, d[3] = {0, 0, 0}, o[3] = {0, 0, 0};
     // particle i's row of slots; an overflowed list is flagged and redone
     const int64_t k0 = sd.nbr0 + (i - sd.p0) * sd.slots;
     const int cnt = live ? min(nstart[i], sd.slots) : 0;
+    T4 next;
+    if (sub < cnt) next = ld_record(geo + k0 + sub);
     for (int n = sub; n < cnt; n += G) {
-      const int64_t k = k0 + n;
-      const T4 gg = geo[k];  // separation x_i - x_j and j, stored by the list build
+      const T4 gg = next;  // separation x_i - x_j and j, stored by the list build
+      if (n + G < cnt) next = ld_record(geo + k0 + n + G);
       const int j = real_as_index<T>(gg.w);
-      const T r2 = gg.x * gg.x + gg.y * gg.y + gg.z * gg.z;
-      const T ir = sizeof(T) == 4 ? (T)rsqrtf((float)r2) : (T)1 / sqrt(r2), r = r2 * ir;
-      T rh[3] = {gg.x * ir, gg.y * ir, gg.z * ir};
-      T f[7];
-      lookup<SHT, MODE>(tab, a, r, f);
       T4 q0, q1;
       if constexpr (sizeof(T) == 4) ldg8((const float *)vcell + 8 * (size_t)j, q0, q1);  // the 8 slots of row j
       else q0 = vc4[2 * j], q1 = vc4[2 * j + 1];
-      T s[5] = {q0.w, q1.x, q1.y, q1.z, q1.w};
-      T v[3];
-      Smul(s, rh, v);
-      const T q = rh[0] * v[0] + rh[1] * v[1] + rh[2] * v[2];
-      const T F[3] = {q0.x, q0.y, q0.z};
-      const T rf = HAS_F ? rh[0] * F[0] + rh[1] * F[1] + rh[2] * F[2] : (T)0;
-      // the terms of each output along the same direction are collected first:
-      // U = f2 v + f0 F + (f3 q + (f1 - f0) rf) rh;
-      // E = f4 s + Y(f5 v - f2 F / 2, rh) + (f6 q - f3 rf) / 2 Y(rh, rh)
-      // (Y(., rh) is linear in its first argument)
-      if (WANT_U) {
-        T c = f[3] * q;
-        if (HAS_F) c += (f[1] - f[0]) * rf;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) U[m] += f[2] * v[m] + c * rh[m] + (HAS_F ? f[0] * F[m] : (T)0);
+      const T r2 = gg.x * gg.x + gg.y * gg.y + gg.z * gg.z;
+      const T ir = sizeof(T) == 4 ? (T)fast_rsqrt((float)r2) : (T)1 / sqrt(r2), r = r2 * ir;
+      const T rh[3] = {gg.x * ir, gg.y * ir, gg.z * ir};
+      T f[7];
+      if (LK == LK_POLY && (float)r2 >= poly.r02) {
+        const float t = fmaf(poly.ta, (float)ir, poly.tb), dr = (float)r - poly.r0, g = fast_exp2(-poly.cg * dr * dr);
+        if (HAS_F) f[0] = (T)(g * poly_at(poly, 0, t));
+        if (HAS_F) f[1] = (T)(g * poly_at(poly, 1, t));
+        if (WANT_U || HAS_F) f[2] = (T)(g * poly_at(poly, 2, t));
+        if (WANT_U || HAS_F) f[3] = (T)(g * poly_at(poly, 3, t));
+        if (WANT_E) {
+          f[4] = (T)(g * poly_at(poly, 4, t));
+          f[5] = (T)(g * poly_at(poly, 5, t));
+          f[6] = (T)(g * poly_at(poly, 6, t));
+        }
+      } else {
+        lookup<LK == LK_SMEM, MODE>(tab, a, r, f);
+        if (HAS_F) f[1] -= f[0];
       }
-      if (WANT_E) {
-        T pv[3], sy[5], yr[5];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) pv[m] = f[5] * v[m] - (HAS_F ? (T)0.5 * f[2] * F[m] : (T)0);
-        symY(pv, rh, sy);
-        symY(rh, rh, yr);  // = 2 y(rh)
-        const T cy = (T)0.5 * (f[6] * q - (HAS_F ? f[3] * rf : (T)0));
-#pragma unroll
-        for (int m = 0; m < 5; ++m) E[m] += f[4] * s[m] + sy[m] + cy * yr[m];
-      }
+      const T row[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+      pair_terms<T, MODE>(rh, row, f, U, d, o);
     }
+    const T r2 = (T)1.4142135623730951;
+    T E[5] = {r2 * (d[0] - d[1]), (T)0.81649658092772603 * (d[0] + d[1] - 2 * d[2]), r2 * o[0], r2 * o[1], r2 * o[2]};
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
+    for (int s = G / 2; s > 0; s >>= 1) {
 #pragma unroll
-      for (int m = 0; m < 3; ++m) U[m] += __shfl_xor_sync(0xffffffffu, U[m], o, G);
+      for (int m = 0; m < 3; ++m)
+        if (WANT_U) U[m] += __shfl_xor_sync(0xffffffffu, U[m], s, G);
 #pragma unroll
-      for (int m = 0; m < 5; ++m) E[m] += __shfl_xor_sync(0xffffffffu, E[m], o, G);
+      for (int m = 0; m < 5; ++m)
+        if (WANT_E) E[m] += __shfl_xor_sync(0xffffffffu, E[m], s, G);
     }
     if (live && sub == 0) {
       T4 s0 = v4[2 * i], s1 = v4[2 * i + 1];
@@ -211,36 +290,40 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (SHT ? 1 : 4) : 1) k_real
   });
 }
 
-template <typename T, int MODE, int G>
-void launch_real_m(pse_ctx *c, const RealArgs &a, const void *vin, void *vout, cudaStream_t s) {
-  const size_t tab_bytes = sizeof(T) * 8 * (size_t)a.len;
-  if (sizeof(T) == 4 && c->real_smem_table && tab_bytes <= c->smem_optin) {
-    auto kern = k_real<T, MODE, G, true>;
+template <typename T, int MODE, int G, int LK>
+void launch_real_k(pse_ctx *c, const RealArgs &a, const void *vin, void *vout, const void *tab, cudaStream_t s) {
+  constexpr int NT = LK == LK_SMEM ? 1024 : 256;
+  auto kern = k_real<T, MODE, G, LK>;
+  const size_t sm = LK == LK_SMEM ? sizeof(T) * 8 * (size_t)a.len : 0;
+  if (LK == LK_SMEM) {
     static std::once_flag once;
     std::call_once(once, [&] {
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_optin);
       cudaGetLastError();
     });
-    static std::atomic<int> per_sm{0};
-    const int64_t items = ceil_div(a.Ntot * G, 1024);
-    unsigned grid = persistent_grid(c, kern, 1024, tab_bytes, items, per_sm);
-    int *q = next_queue(c);
-    kern<<<grid, 1024, tab_bytes, s>>>(a, c->d_sys, c->d_p0, c->d_active, q, (int)items, c->d_nbr_start,
-                                       (const typename V4<T>::t *)c->d_nbr_geo, (const T *)vin,
-                                       (const T *)c->d_vcell, (T *)vout, (const T *)c->d_table);
-    return;
   }
-  auto kern = k_real<T, MODE, G>;
   static std::atomic<int> per_sm{0};
-  const int64_t items = ceil_div(a.Ntot * G, 256);
-  const void *tab = c->d_table;  // FP32 partial products: their interval table
-  if (sizeof(T) == 4 && MODE == M_SE) tab = c->d_table_e;
-  if (sizeof(T) == 4 && (MODE == M_FSU || MODE == M_SU)) tab = c->d_table_u;
-  unsigned grid = persistent_grid(c, kern, 256, 0, items, per_sm);
+  const int64_t items = ceil_div(a.Ntot * G, NT);
+  const unsigned grid = persistent_grid(c, kern, NT, sm, items, per_sm);
   int *q = next_queue(c);
-  kern<<<grid, 256, 0, s>>>(a, c->d_sys, c->d_p0, c->d_active, q, (int)items, c->d_nbr_start,
-                            (const typename V4<T>::t *)c->d_nbr_geo, (const T *)vin, (const T *)c->d_vcell,
-                            (T *)vout, (const T *)tab);
+  kern<<<grid, NT, sm, s>>>(a, c->poly, c->d_sys, c->d_p0, c->d_active, q, (int)items, c->d_nbr_start,
+                            (const typename V4<T>::t *)c->d_nbr_geo, (const T *)vin, (const T *)c->d_vcell, (T *)vout,
+                            (const T *)tab);
+}
+
+// FP32: the table in shared memory where the autotuner chose it, else the polynomial fit
+// where it holds (RealPoly::ok), else the table; the partial products read their interval
+// tables.
+template <typename T, int MODE, int G>
+void launch_real_m(pse_ctx *c, const RealArgs &a, const void *vin, void *vout, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4) {
+    if (c->real_smem_table && sizeof(T) * 8 * (size_t)a.len <= c->smem_optin)
+      return launch_real_k<T, MODE, G, LK_SMEM>(c, a, vin, vout, c->d_table, s);
+    const void *tab = MODE == M_SE ? c->d_table_e : (MODE == M_FULL ? c->d_table : c->d_table_u);
+    if (c->poly.ok) return launch_real_k<T, MODE, G, LK_POLY>(c, a, vin, vout, tab, s);
+    return launch_real_k<T, MODE, G, LK_TABLE>(c, a, vin, vout, tab, s);
+  }
+  launch_real_k<T, MODE, G, LK_TABLE>(c, a, vin, vout, c->d_table, s);
 }
 
 template <typename T, int G>
@@ -289,8 +372,8 @@ __device__ __forceinline__ void rot_lookup(const double *tab, const RealArgs &a,
   else b = max(b, a.k2);
   b = max(0, min(b, a.len - 4));
   double t = x - (double)b;
-  double w0 = -(t - 1) * (t - 2) * (t - 3) / 6.0, w1 = t * (t - 2) * (t - 3) / 2.0;
-  double w2 = -t * (t - 1) * (t - 3) / 2.0, w3 = t * (t - 1) * (t - 2) / 6.0;
+  const double c6 = 1.0 / 6.0, u0 = t * (t - 1), u1 = (t - 2) * (t - 3);
+  const double w0 = -c6 * (t - 1) * u1, w1 = 0.5 * t * u1, w2 = -0.5 * u0 * (t - 3), w3 = c6 * u0 * (t - 2);
   const double *r0 = tab + 4 * (size_t)b;
 #pragma unroll
   for (int k = 0; k < 3; ++k)
@@ -390,15 +473,17 @@ __global__ void k_cell_gather12(int64_t N, const int *__restrict__ list, const T
   vcell[e] = vin[12 * (int64_t)list[k] + (e - 12 * k)];
 }
 
-// vcell[k] = vin[list[k]]: the 8-real rows of the input vector in cell-list order.
+// vcell[k] = cell_row(vin[list[k]]): the rows of the input vector in cell-list order.
 template <typename T>
 __global__ void k_cell_gather(int64_t N, const int *__restrict__ list, const typename V4<T>::t *__restrict__ vin,
                               typename V4<T>::t *__restrict__ vcell) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= N) return;
   const int64_t j = list[k];
-  vcell[2 * k] = vin[2 * j];
-  vcell[2 * k + 1] = vin[2 * j + 1];
+  typename V4<T>::t lo, hi;
+  load_row(vin, j, lo, hi);
+  cell_row(lo, hi);
+  store_row(vcell, k, lo, hi);
 }
 
 // Harmonic overlap repulsion F_i = sum_j k (2a - r_ij) rh_ij over neighbours

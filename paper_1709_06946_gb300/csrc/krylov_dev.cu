@@ -365,22 +365,27 @@ __global__ void k_kr_finish(KrArgs a, const T *__restrict__ rows, T *w, int cap,
 // particle's place in that list).
 template <typename T>
 __global__ void k_kr_next(KrArgs a, T *basis, const T *src, T *vin, T *vcell, const int *__restrict__ pos) {
-  using V = V16<T>;
-  using VT = typename V::t;
+  using T4 = typename V4<T>::t;
   const Chunk ch = chunk_of(a.va);
   if (!a.va.active[ch.s]) return;
   const T f = (T)a.k.coef[(size_t)ch.s * COEF_STRIDE + CO_FAC];
   T *dst = basis + (int64_t)*a.k.iter * a.stride;
-  for (int64_t e = ch.beg + (int64_t)threadIdx.x * V::n; e < ch.end; e += (int64_t)blockDim.x * V::n) {
-    const int64_t p = pos[e >> 3];
-    T x[V::n];
-    V::get(*(const VT *)(src + e), x);
-#pragma unroll
-    for (int i = 0; i < V::n; ++i) x[i] *= f;
-    const VT v = V::put(x);
-    *(VT *)(dst + e) = v;
-    *(VT *)(vin + e) = v;
-    *(VT *)(vcell + 8 * p + (e & 7)) = v;
+  for (int64_t i = ch.beg / 8 + threadIdx.x; i < ch.end / 8; i += blockDim.x) {  // a row of 8 per thread
+    const int64_t p = pos[i];
+    T4 lo, hi;
+    load_row((const T4 *)src, i, lo, hi);
+    lo.x *= f;
+    lo.y *= f;
+    lo.z *= f;
+    lo.w *= f;
+    hi.x *= f;
+    hi.y *= f;
+    hi.z *= f;
+    hi.w *= f;
+    store_row((T4 *)dst, i, lo, hi);
+    store_row((T4 *)vin, i, lo, hi);
+    cell_row(lo, hi);
+    store_row((T4 *)vcell, p, lo, hi);
   }
 }
 

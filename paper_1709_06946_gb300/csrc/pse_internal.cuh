@@ -60,6 +60,21 @@ struct RealTable {
   std::vector<double> v;   // len x 8
 };
 void build_real_table(const Params &p, int points_per_2a, RealTable &t);
+// FP32 fit of the seven functions on [2a, r_cut]: f_k(r) = exp2(-cg (r - r0)^2) P_k(ta / r + tb)
+// with r0 = 2a and exp(-xi^2 (r - 2a)^2) the decay of the screened functions, f_1 - f_0
+// in place of f_1.  Degree 8 is off by 5e-7 of each function's maximum at xi = 0.5, where
+// linear interpolation of the table is off by up to 9e-6; ok = 0 where the fit is not the
+// closer of the two for every function (xi below about 0.35 / a) or the caller set the
+// table's density (option table_points).
+constexpr int POLY_DEG = 8;
+struct RealPoly {
+  int ok = 0;
+  float ta = 0, tb = 0, r0 = 0, r02 = 0, cg = 0;
+  float c[7][POLY_DEG + 1] = {};
+};
+// Fits the nodes of t beyond contact; returns the largest ratio over the functions of the
+// fit's error to that of the table's linear interpolation there.
+double build_real_poly(const Params &p, const RealTable &t, RealPoly &f);
 // The same table rounded to FP32 into a caller buffer of len x 8 floats (no allocation).
 void fill_real_table_f32(const Params &p, int points_per_2a, int len, float *out, double *self_uf,
                          double *self_es);
@@ -219,6 +234,7 @@ struct pse_ctx {
   // FP32 interval tables for the partial products: per interval q the values at
   // q and q + 1 of f4..f6 (S -> E) or of f0..f3 ([F; S] -> U), 8 floats each
   void *d_table_e = nullptr, *d_table_u = nullptr;
+  pse::RealPoly poly;           // FP32 fit of the scalar functions beyond contact
   int table_len = 0, table_k2 = 0;
   double table_dr = 0, self_uf = 0, self_es = 0;
 

@@ -497,6 +497,106 @@ void build_real_table(const Params &p, int points_per_2a, RealTable &t) {
   }
 }
 
+double build_real_poly(const Params &p, const RealTable &t, RealPoly &f) {
+  constexpr int D = POLY_DEG, NB = D + 1;
+  const double r0 = 2.0 * p.a, rc = std::max(p.rcut, 1.05 * r0), u0 = 1.0 / rc, u1 = 1.0 / r0;
+  const double ta = 2.0 / (u1 - u0), tb = -(u1 + u0) / (u1 - u0);
+  f.r0 = (float)r0;
+  f.r02 = (float)(r0 * r0 * (1.0 + 1e-6));  // at contact the table, which ends there exactly
+  f.ta = (float)ta;
+  f.tb = (float)tb;
+  f.cg = (float)(p.xi * p.xi * 1.4426950408889634);
+  // sample points: table nodes from contact to r_cut, about 500 of them, the ends included
+  std::vector<int> node;
+  const int last = std::min(t.len - 1, (int)std::floor(rc / t.dr));
+  if (last - t.k2 < 4 * NB) return HUGE_VAL;
+  const int step = std::max(1, (last - t.k2) / 500);
+  for (int i = t.k2; i < last; i += step) node.push_back(i);
+  node.push_back(last);
+  const int n = (int)node.size();
+  std::vector<double> B((size_t)n * NB), g(n), y(n), w(n), e(n);
+  for (int q = 0; q < n; ++q) {
+    const double r = node[q] * t.dr, x = ta / r + tb;
+    g[q] = std::exp(-p.xi * p.xi * (r - r0) * (r - r0));
+    B[(size_t)q * NB] = 1.0;
+    B[(size_t)q * NB + 1] = x;
+    for (int d = 2; d < NB; ++d) B[(size_t)q * NB + d] = 2 * x * B[(size_t)q * NB + d - 1] - B[(size_t)q * NB + d - 2];
+  }
+  auto value = [&](int i, int k) { return t.v[(size_t)i * 8 + k] - (k == 1 ? t.v[(size_t)i * 8] : 0.0); };
+  double worst = 0.0;
+  for (int k = 0; k < 7; ++k) {
+    for (int q = 0; q < n; ++q) y[q] = value(node[q], k);
+    double table = 0.0;  // error of linear interpolation, an eighth of the second difference
+    for (int i = t.k2 + 1; i < last; ++i)
+      table = std::max(table, std::fabs(value(i - 1, k) - 2.0 * value(i, k) + value(i + 1, k)) / 8.0);
+    // Lawson's iteration: least squares with weights that grow where the error is large
+    // tends to the minimax fit; g weighs the error of P back to that of f
+    std::fill(w.begin(), w.end(), 1.0);
+    double best = HUGE_VAL, cheb[NB] = {0};
+    for (int it = 0; it < 30; ++it) {
+      double M[NB][NB + 1] = {};
+      for (int q = 0; q < n; ++q) {
+        const double *b = &B[(size_t)q * NB], wg = w[q] * g[q];
+        for (int i = 0; i < NB; ++i) {
+          for (int j = i; j < NB; ++j) M[i][j] += wg * g[q] * b[i] * b[j];
+          M[i][NB] += wg * b[i] * y[q];
+        }
+      }
+      for (int i = 0; i < NB; ++i)
+        for (int j = 0; j < i; ++j) M[i][j] = M[j][i];
+      for (int i = 0; i < NB; ++i) {  // Gaussian elimination with row exchanges
+        int piv = i;
+        for (int r = i + 1; r < NB; ++r)
+          if (std::fabs(M[r][i]) > std::fabs(M[piv][i])) piv = r;
+        for (int c = 0; c <= NB; ++c) std::swap(M[i][c], M[piv][c]);
+        if (M[i][i] == 0.0) return HUGE_VAL;
+        for (int r = i + 1; r < NB; ++r) {
+          const double m = M[r][i] / M[i][i];
+          for (int c = i; c <= NB; ++c) M[r][c] -= m * M[i][c];
+        }
+      }
+      double cf[NB];
+      for (int i = NB - 1; i >= 0; --i) {
+        double s = M[i][NB];
+        for (int j = i + 1; j < NB; ++j) s -= M[i][j] * cf[j];
+        cf[i] = s / M[i][i];
+      }
+      double big = 0.0;
+      for (int q = 0; q < n; ++q) {
+        double s = 0.0;
+        for (int d = 0; d < NB; ++d) s += cf[d] * B[(size_t)q * NB + d];
+        e[q] = std::fabs(s * g[q] - y[q]);
+        big = std::max(big, e[q]);
+      }
+      if (big < best) {
+        best = big;
+        std::copy(cf, cf + NB, cheb);
+      }
+      double wmax = 0.0;
+      for (int q = 0; q < n; ++q) {
+        w[q] *= e[q] / big + 1e-3;
+        wmax = std::max(wmax, w[q]);
+      }
+      for (int q = 0; q < n; ++q) w[q] /= wmax;
+    }
+    // Chebyshev series to powers of t
+    double pw[NB] = {0}, T0[NB] = {1.0}, T1[NB] = {0.0, 1.0};
+    for (int d = 0; d < NB; ++d) {
+      const double *Td = d == 0 ? T0 : T1;
+      for (int i = 0; i < NB; ++i) pw[i] += cheb[d] * Td[i];
+      if (d >= 1) {
+        double T2[NB];
+        for (int i = 0; i < NB; ++i) T2[i] = (i > 0 ? 2 * T1[i - 1] : 0.0) - T0[i];
+        std::copy(T1, T1 + NB, T0);
+        std::copy(T2, T2 + NB, T1);
+      }
+    }
+    for (int d = 0; d < NB; ++d) f.c[k][d] = (float)pw[d];
+    worst = std::max(worst, table > 0 ? best / table : HUGE_VAL);
+  }
+  return worst;
+}
+
 void fill_real_table_f32(const Params &p, int points_per_2a, int len, float *out, double *self_uf,
                          double *self_es) {
   static const GL gl(40);
@@ -551,6 +651,30 @@ int pse_internal_real_functions(double a, double eta, double xi, int n, const do
     self2[1] = t.self_es;
   }
   return 0;
+}
+
+// The FP32 fit of the seven functions (f1 - f0 in place of f1) at separations r[0..n)
+// beyond contact, evaluated as the pair sum does (out: n x 7); returns
+// build_real_poly's ratio of errors.
+double pse_internal_real_poly(double a, double eta, double xi, double rcut, int n, const float *r, float *out) {
+  pse::Params p{};
+  p.a = a;
+  p.eta = eta;
+  p.xi = xi;
+  p.rcut = rcut;
+  pse::RealTable t;
+  pse::RealPoly f;
+  pse::build_real_table(p, 1024, t);
+  const double err = pse::build_real_poly(p, t, f);
+  for (int i = 0; i < n; ++i) {
+    const float x = std::fmaf(f.ta, 1.0f / r[i], f.tb), dr = r[i] - f.r0, g = std::exp2(-f.cg * dr * dr);
+    for (int k = 0; k < 7; ++k) {
+      float v = f.c[k][pse::POLY_DEG];
+      for (int d = pse::POLY_DEG - 1; d >= 0; --d) v = std::fmaf(v, x, f.c[k][d]);
+      out[7 * (size_t)i + k] = g * v;
+    }
+  }
+  return err;
 }
 
 // Spreading tile for a grid of Ng points per side, support P and real size ts
