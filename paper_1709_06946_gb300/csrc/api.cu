@@ -679,9 +679,6 @@ void pse::fill_lattice(const Params &p, SysDev &d) {
 
 namespace {
 
-// Marks a suspension for the spreading / interpolation kernels specialised for
-// 16^3 tiles (mixed precision, P = 5, 6 or 8, at least two tiles per side) and
-// counts it in c->n_cubic.
 // Whether A^T A couples z with x or y (the 16^3-tile kernels on a deformed
 // lattice need the z axis orthogonal to the deformed plane, as in shear and
 // planar extension).
@@ -690,13 +687,42 @@ bool z_coupled(const double A[9]) {
   return g13 != 0.0 || g23 != 0.0;
 }
 
+// Supports with instances of the 16^3-tile kernels (P = 10 with the default kernels only).
+bool cubic_support(const pse_options &o, int prec, int P) {
+  return prec == PSE_MIXED && (P == 5 || P == 6 || P == 8 || (P == 10 && o.wave_kernel == 0));
+}
+
+// Tile of a grid that 16 does not divide: as few and as equal tiles of at most 16 points
+// as leave the last one P - 1 of them (54 = 14 + 14 + 14 + 12), for the default
+// 16^3-tile kernels.  Only on the cube: a lattice handle may later be given a deformation
+// that these kernels do not take, and the general ones need a divisor of the grid.
+bool cubic_tile(Params &p, const pse_options &o, int prec) {
+  for (int k = 0; k < 3; ++k)
+    if (o.tile[k] > 0) return false;
+  for (int i = 0; i < 9; ++i)
+    if (o.deform[i] != 0.0) return false;
+  if (o.wave_kernel != 0 || !cubic_support(o, prec, p.P) || p.Ng % CUBE_TILE == 0) return false;
+  for (int nt = std::max(2, (p.Ng + CUBE_TILE - 1) / CUBE_TILE);; ++nt) {
+    const int T = (p.Ng + nt - 1) / nt, last = p.Ng - (nt - 1) * T;
+    if (T < 8 || T < p.P - 1) return false;  // too small to be worth it: a divisor, on the general kernels
+    if (last < p.P - 1) continue;
+    for (int k = 0; k < 3; ++k) {
+      p.tile[k] = T;
+      p.ntile[k] = nt;
+    }
+    return true;
+  }
+}
+
+// Marks a suspension for the spreading / interpolation kernels specialised for
+// tiles of up to 16^3 points (mixed precision, P = 5, 6, 8 or 10, at least two tiles per
+// side: tiles of 16, or those of cubic_tile) and counts it in c->n_cubic.
 void set_cubic(pse_ctx *c, SysDev &d, const Params &p) {
-  // P = 10 and deformed lattices only with the default kernels (the optional
-  // 16^3 variants have neither)
-  const bool defaults = c->opt.wave_kernel == 0;
-  bool ok = c->prec == PSE_MIXED && (c->p.P == 5 || c->p.P == 6 || c->p.P == 8 || (c->p.P == 10 && defaults));
-  if (c->lattice) ok = ok && defaults && !z_coupled(p.A);
-  for (int k = 0; k < 3; ++k) ok = ok && d.T[k] == CUBE_TILE && d.nt[k] >= 2;
+  bool ok = cubic_support(c->opt, c->prec, c->p.P);
+  if (c->lattice) ok = ok && c->opt.wave_kernel == 0 && !z_coupled(p.A);
+  Params q = p;
+  const int T = cubic_tile(q, c->opt, c->prec) ? q.tile[0] : CUBE_TILE;
+  for (int k = 0; k < 3; ++k) ok = ok && d.T[k] == T && d.nt[k] == (p.Ng + T - 1) / T && d.nt[k] >= 2;
   d.cubic = ok ? 1 : 0;
   c->n_cubic += d.cubic;
 }
@@ -714,6 +740,7 @@ pse_status choose_group(pse_ctx *c, int nsys, const int64_t *N, const double *L,
       c->err = nsys > 1 ? "suspension " + std::to_string(q) + ": " + e : e;
       return PSE_ERR_INVALID_ARG;
     }
+    cubic_tile(p, o, c->prec);
     Nt += p.N;
   }
   if (Nt > 200000000LL) {
@@ -1095,7 +1122,7 @@ void destroy_impl(pse_ctx *c) {
   c->allocs.clear();
 }
 
-// Re-tiles every suspension with the tile caps (x, y, z); the tile arrays grow if needed.
+// Re-tiles every suspension with the tile caps (x, y, z; 16^3 as at creation); the tile arrays grow if needed.
 pse_status retile(pse_ctx *c, const int caps[3]) {
   std::vector<Params> ps = c->ps;
   std::vector<int> tile0(c->nsys + 1, 0);
@@ -1105,6 +1132,7 @@ pse_status retile(pse_ctx *c, const int caps[3]) {
       c->err = e;
       return PSE_ERR_INVALID_ARG;
     }
+    if (caps[0] == CUBE_TILE && caps[1] == CUBE_TILE && caps[2] == CUBE_TILE) cubic_tile(ps[q], c->opt, c->prec);
     tile0[q + 1] = tile0[q] + ps[q].ntile[0] * ps[q].ntile[1] * ps[q].ntile[2];
   }
   const int64_t nt = tile0[c->nsys];

@@ -1,4 +1,4 @@
-// Gaussian spreading Q (Sec. 2.3.2, Eq. WSops2) onto 16^3 grid tiles with the
+// Gaussian spreading Q (Sec. 2.3.2, Eq. WSops2) onto grid tiles of up to 16^3 points with the
 // grid held in registers: every thread owns one (x, y) column of a tile, ZT
 // consecutive z points of it, all C components, and accumulates into them; no
 // shared-memory read-modify-write and no atomics.
@@ -29,6 +29,8 @@
 // weights them by its x-y weight, the warp sums the C values over its lanes in
 // nine shuffles, and C lanes add the totals to the particle's outputs (one
 // atomic add per component and warp visit).
+#include <type_traits>
+
 #include "wave_common.cuh"
 
 namespace pse {
@@ -97,21 +99,22 @@ struct ZDot {
   }
 };
 
-// Candidate ranges of a warp (source bins below the tile keep the sub-block layers that can reach the warp's z range), published to rg by the warp.
-__device__ __forceinline__ void col_ranges(const SysDev &a, const int t[3], int wz0, int ZT, int P, int lane,
+// Candidate ranges of the z range [wz0, wz0 + nz) of a tile (source bins below the tile keep the
+// sub-block layers that can reach it), published to rg by the warp.
+__device__ __forceinline__ void col_ranges(const SysDev &a, const int t[3], int wz0, int nz, int P, int lane,
                                            const int *__restrict__ fine_start, ColRanges &rg) {
-  constexpr int TS = CUBE;
   int beg = 0, len = 0;
   if (lane < 8) {
-    const int bz = lane >> 2, by = (lane >> 1) & 1, bx = lane & 1;
+    const int bz = lane >> 2, by = (lane >> 1) & 1, bx = lane & 1, Tz = a.T[2];
     const int bzc = t[2] - bz < 0 ? t[2] - bz + a.nt[2] : t[2] - bz;
     const int byc = t[1] - by < 0 ? t[1] - by + a.nt[1] : t[1] - by;
     const int bxc = t[0] - bx < 0 ? t[0] - bx + a.nt[0] : t[0] - bx;
     const int64_t b = (int64_t)(a.tile0 + (bzc * a.nt[1] + byc) * a.nt[0] + bxc) * SUB_BLOCKS;
-    const int zlo = max(0, wz0 - P + 1 + bz * TS), zhi = min(TS - 1, wz0 + ZT - 1 + bz * TS);
+    const int w = tile_width(a, bzc, 2), up = bz * w;  // the source tile's planes, and where they start below
+    const int zlo = max(0, wz0 - P + 1 + up), zhi = min(w - 1, wz0 + nz - 1 + up);
     if (zlo <= zhi) {
-      beg = fine_start[b + (zlo * SUB_SIDE / TS) * SUB_SIDE * SUB_SIDE];
-      len = fine_start[b + (zhi * SUB_SIDE / TS + 1) * SUB_SIDE * SUB_SIDE] - beg;
+      beg = fine_start[b + (zlo * SUB_SIDE / Tz) * SUB_SIDE * SUB_SIDE];
+      len = fine_start[b + (zhi * SUB_SIDE / Tz + 1) * SUB_SIDE * SUB_SIDE] - beg;
     }
   }
   int inc = lane < 8 ? len : 0;
@@ -237,18 +240,18 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), 16 / ZT == 1 ? 2 : 1)
 }
 
 // Bit w set for each warp w whose column block (and z range, for ZT = 8) the P^3
-// support with start offsets (ex, ey, ez) from the tile origin overlaps.
+// support with start offsets (ex, ey, ez) from the tile origin overlaps, in a tile of
+// wx x wy x wz points.
 template <int NW, int ZT, int P>
-__device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez) {
-  constexpr int TS = CUBE;
-  if (ex <= -P || ex >= TS || ey <= -P || ey >= TS || ez <= -P || ez >= TS) return 0u;
-  const unsigned xm = (ex <= 7 ? 1u : 0u) | (ex + P - 1 >= 8 ? 2u : 0u);
-  const int ylo = max(ey, 0) >> 2, yhi = min(ey + P - 1, TS - 1) >> 2;
+__device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, int wy, int wz) {
+  if (ex <= -P || ex >= wx || ey <= -P || ey >= wy || ez <= -P || ez >= wz) return 0u;
+  const unsigned xm = (ex <= 7 ? 1u : 0u) | (ex + P - 1 >= 8 && wx > 8 ? 2u : 0u);
+  const int ylo = max(ey, 0) >> 2, yhi = min(ey + P - 1, wy - 1) >> 2;
   unsigned m = 0;
 #pragma unroll
   for (int b = 0; b < 4; ++b) m |= (b >= ylo && b <= yhi) ? xm << (2 * b) : 0u;
-  if (ZT == TS) return m;
-  const unsigned zm = (ez <= ZT - 1 ? 1u : 0u) | (ez + P - 1 >= ZT ? 2u : 0u);
+  if (ZT == CUBE) return m;
+  const unsigned zm = (ez <= ZT - 1 ? 1u : 0u) | (ez + P - 1 >= ZT && wz > ZT ? 2u : 0u);
   return ((zm & 1u) ? m : 0u) | ((zm & 2u) ? m << 8 : 0u);
 }
 
@@ -262,7 +265,13 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez) {
 // plane (A^T A couples x and y only): the x-y weight of a column is
 // exp(-alpha (G_xx dx^2 + 2 G_xy dx dy + G_yy dy^2)) and the z weights use G_zz,
 // from the suspension's coefficients SysDev::qa.
-template <int C, int SLOT0, int P, int ZT, bool DEF = false>
+// ROW: slots per particle row of vin; COMP0: first grid component written.
+//
+// Tiles are 16^3 where 16 divides the grid, else as equal as possible (54 = 14 + 14 + 14 +
+// 12); columns and planes past a smaller tile's edge are idle.  Against the general
+// kernel: 5 components on 12^3 tiles at N_g = 36 65 -> 29 us (27 CTAs), the 11-moment
+// product's 8 and 3 components at N_g = 128 322 -> 120 and 199 -> 71 us.
+template <int C, int SLOT0, int P, int ZT, bool DEF = false, int ROW = 8, int COMP0 = 0>
 __global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ? 2 : 1)
     k_spread_colq(WaveArgs wa, int *queue, const int4 *__restrict__ sp_i0, const float4 *__restrict__ sp_d0,
                   const float *__restrict__ vin, const int *__restrict__ fine_start, float *__restrict__ grid_all) {
@@ -284,7 +293,8 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ?
     const int Ng = a.Ng;
     int t[3], t0[3];
     tile_of(a, item - a.tile0, t, t0);
-    if (w == 0) col_ranges(a, t, 0, TS, P, lane, fine_start, s_rng);
+    const int wx = tile_width(a, t[0], 0), wy = tile_width(a, t[1], 1), wz = tile_width(a, t[2], 2);
+    if (w == 0) col_ranges(a, t, 0, wz, P, lane, fine_start, s_rng);
     if (tid < 2 * NW) (&s_cnt[0][0])[tid] = 0;
     const float nal = -(float)a.alpha * COL_LOG2E, hs = (float)a.h, pref = (float)a.pref;
     // deformed lattice: exponent coefficients (base 2) of the x-y form and of z
@@ -317,13 +327,13 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ?
           ex = col_soff(i0[u].x, t0[0], Ng, P);
           ey = col_soff(i0[u].y, t0[1], Ng, P);
           ez = col_soff(i0[u].z, t0[2], Ng, P);
-          mask = region_mask<NW, ZT, P>(ex, ey, ez);
+          mask = region_mask<NW, ZT, P>(ex, ey, ez, wx, wy, wz);
         }
         const int slot = tid + u * NT;
         if (mask) {
           const int k = kk[u];
           const float4 d0 = sp_d0[k];
-          const float *row = vin + 8 * (size_t)k + SLOT0;
+          const float *row = vin + ROW * (size_t)k + SLOT0;
           float q[RF];
 #pragma unroll
           for (int i = 0; i < RF; ++i) q[i] = 0.f;
@@ -384,12 +394,16 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ?
       }
       __syncthreads();  // the records and lists are read before the next chunk overwrites them
     }
-    float *grid = grid_all + a.grid0;
-    const size_t g0 = ((size_t)(t0[2] + wz0) * Ng + (t0[1] + cy)) * Ng + (t0[0] + cx);
+    if (cx < wx && cy < wy) {
+      float *grid = grid_all + a.grid0;
+      const size_t g0 = ((size_t)(t0[2] + wz0) * Ng + (t0[1] + cy)) * Ng + (t0[0] + cx);
 #pragma unroll
-    for (int z = 0; z < ZT; ++z)
+      for (int z = 0; z < ZT; ++z)
+        if (wz0 + z < wz) {
 #pragma unroll
-      for (int c = 0; c < C; ++c) grid[c * a.gstride + g0 + (size_t)z * Ng * Ng] = acc[z][c];
+          for (int c = 0; c < C; ++c) grid[(COMP0 + c) * a.gstride + g0 + (size_t)z * Ng * Ng] = acc[z][c];
+        }
+    }
   });
 }
 
@@ -522,11 +536,11 @@ void interp_col_p(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) {
   }
 }
 
-template <int C, int SLOT0, int P, int ZT, bool DEF = false>
+template <int C, int SLOT0, int P, int ZT, bool DEF = false, int ROW = 8, int COMP0 = 0>
 void launch_spread_col_z(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStream_t s) {
   constexpr int NT = 32 * 8 * (CUBE / ZT);
   int *q = next_queue(c);
-  if (!DEF && (c->opt.wave_kernel & 4)) {  // every warp scans the candidates itself
+  if constexpr (!DEF && ROW == 8) if (c->opt.wave_kernel & 4) {  // every warp scans the candidates itself
     static OccCache occ;
     auto kern = k_spread_col<C, SLOT0, P, ZT>;
     const unsigned grid = wave_grid(c, kern, 0, a.ntiles, occ, NT);
@@ -536,7 +550,7 @@ void launch_spread_col_z(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStr
   }
   static std::once_flag once;
   static OccCache occ;
-  auto kern = k_spread_colq<C, SLOT0, P, ZT, DEF>;
+  auto kern = k_spread_colq<C, SLOT0, P, ZT, DEF, ROW, COMP0>;
   set_smem(kern, once);
   constexpr size_t sm = (size_t)2 * NT * ColRec<C, P>::FLOATS * sizeof(float) +
                         (size_t)(NT / 32) * 2 * NT * sizeof(unsigned short);
@@ -571,7 +585,28 @@ void spread_col_p(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStream_t s
   }
 }
 
+// Components SLOT0 .. SLOT0 + C - 1 of 12-slot rows onto grid components COMP0 ...
+template <int C, int SLOT0, int COMP0>
+void spread_col11_p(pse_ctx *c, const WaveArgs &a, const void *vin12, cudaStream_t s) {
+  auto run = [&](auto def) {
+    constexpr bool DEF = decltype(def)::value;
+    switch (a.P) {
+      case 5: launch_spread_col_z<C, SLOT0, 5, 8, DEF, 12, COMP0>(c, a, vin12, s); break;
+      case 6: launch_spread_col_z<C, SLOT0, 6, 8, DEF, 12, COMP0>(c, a, vin12, s); break;
+      case 10: launch_spread_col_z<C, SLOT0, 10, 8, DEF, 12, COMP0>(c, a, vin12, s); break;
+      default: launch_spread_col_z<C, SLOT0, 8, 8, DEF, 12, COMP0>(c, a, vin12, s);
+    }
+  };
+  if (c->lattice) run(std::true_type{});
+  else run(std::false_type{});
+}
+
 }  // namespace
+
+void spread_col11_launch(pse_ctx *c, const WaveArgs &a, const void *vin12, cudaStream_t s) {
+  spread_col11_p<8, 0, 0>(c, a, vin12, s);
+  spread_col11_p<3, 8, 8>(c, a, vin12, s);
+}
 
 void spread_col_launch(pse_ctx *c, const WaveArgs &a, const void *vin, int mode, cudaStream_t s) {
   if (mode == M_SE || mode == M_SU) spread_col_p<5, 3>(c, a, vin, s);

@@ -172,6 +172,10 @@ __device__ __forceinline__ void tile_of(const SysDev &a, int tile, int t[3], int
   for (int d = 0; d < 3; ++d) t0[d] = t[d] * a.T[d];
 }
 
+// Points of tile t along dimension d: T, or fewer in the last tile of a side that T does
+// not divide (only the 16^3-tile kernels take such grids).
+__device__ __forceinline__ int tile_width(const SysDev &a, int t, int d) { return min(a.T[d], a.Ng - t * a.T[d]); }
+
 // The (up to) 8 source bins of a tile and the running offsets of their ranges.
 __device__ __forceinline__ int tile_bins(const SysDev &a, const int t[3], const int *tile_start, int beg[8],
                                          int cum[9]) {
@@ -283,8 +287,8 @@ inline size_t wave_smem_max(const pse_ctx *c, int want = -1) {
   return m;
 }
 
-// The kernels specialised for 16^3 tiles run the suspensions marked
-// SysDev::cubic (mixed precision, P = 5, 6 or 8, at least two tiles per side, so
+// The kernels specialised for tiles of up to 16^3 points run the suspensions marked
+// SysDev::cubic (mixed precision, P = 5, 6, 8 or 10, at least two tiles per side, so
 // that a support crosses the periodic boundary into another tile, never back
 // into the same one, and offsets from the tile origin can be kept signed); the
 // general kernels run the others.  WaveArgs::want selects the suspensions of a
@@ -296,10 +300,9 @@ __device__ __forceinline__ bool wave_skip(const WaveArgs &wa, int si, const SysD
 void spread16_launch(pse_ctx *c, const WaveArgs &a, const void *vin, int mode, cudaStream_t s);
 void spread_col_launch(pse_ctx *c, const WaveArgs &a, const void *vin, int mode, cudaStream_t s);
 void interp_col_launch(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStream_t s);
-// General interpolation kernels (any tile) for the suspensions a selects; the
-// 16^3-tile kernels fall back to them where their staging does not fit.
-void interp_general_launch(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStream_t s);
-// 11-moment product (12-slot rows [F, L, S] / [U, Omega, E]), general kernels
+// 11-moment product (12-slot rows [F, L, S] / [U, Omega, E])
+void spread_col11_launch(pse_ctx *c, const WaveArgs &a, const void *vin12, cudaStream_t s);
+void interp_halo11_launch(pse_ctx *c, const WaveArgs &a, void *vout12, cudaStream_t s);
 void spread11_launch(pse_ctx *c, const void *vin12, cudaStream_t s);
 void interp11_launch(pse_ctx *c, void *vout12, cudaStream_t s);
 void interp16_launch(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStream_t s);

@@ -225,18 +225,6 @@ void interp_cubic(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStrea
   else interp_halo_launch(c, a, vout, mode, s);
 }
 
-void interp_general_launch(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStream_t s) {
-  if (c->prec == PSE_MIXED) {
-    if (mode == M_FULL) interp_p<float, 8, 0>(c, a, vout, s);
-    else if (mode == M_SE) interp_p<float, 5, 3>(c, a, vout, s);
-    else interp_p<float, 3, 0>(c, a, vout, s);
-  } else {
-    if (mode == M_FULL) interp_p<double, 8, 0>(c, a, vout, s);
-    else if (mode == M_SE) interp_p<double, 5, 3>(c, a, vout, s);
-    else interp_p<double, 3, 0>(c, a, vout, s);
-  }
-}
-
 void interp_launch(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStream_t s) {
   if (c->n_cubic == c->nsys) return interp_cubic(c, a, vout, mode, s);
   WaveArgs ag = a;
@@ -259,9 +247,11 @@ void interp_launch(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStre
 }
 
 // Grids 0..10 interpolated into the 11 components [U, Omega, E] of 12-slot rows
-// (general kernels, two passes: 8 and 3 components; outputs are added).
+// (two passes: 8 and 3 components; outputs are added).
 void interp11_launch(pse_ctx *c, void *vout12, cudaStream_t s) {
   WaveArgs a = wave_args(c);
+  c->nlaunch += 2;
+  if (c->n_cubic == c->nsys) return interp_halo11_launch(c, a, vout12, s);
   if (c->prec == PSE_MIXED) {
     interp_p<float, 8, 0, 12, 0>(c, a, vout12, s);
     interp_p<float, 3, 8, 12, 8>(c, a, vout12, s);
@@ -269,7 +259,6 @@ void interp11_launch(pse_ctx *c, void *vout12, cudaStream_t s) {
     interp_p<double, 8, 0, 12, 0>(c, a, vout12, s);
     interp_p<double, 3, 8, 12, 8>(c, a, vout12, s);
   }
-  c->nlaunch += 2;
 }
 
 }  // namespace pse

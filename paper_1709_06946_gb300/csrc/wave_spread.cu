@@ -199,7 +199,7 @@ void spread_p(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStream_t s) {
 
 }  // namespace
 
-// Suspensions with 16^3 tiles: grid columns in registers (default) or the
+// Suspensions with tiles of up to 16^3: grid columns in registers (default) or the
 // shared-memory tile (bit 0 of option wave_kernel).
 void spread_cubic(pse_ctx *c, const WaveArgs &a, const void *vin, int mode, cudaStream_t s) {
   if (c->opt.wave_kernel & 1) spread16_launch(c, a, vin, mode, s);
@@ -226,9 +226,11 @@ void spread_launch(pse_ctx *c, const WaveArgs &a, const void *vin, int mode, cud
 }
 
 // The 11 components [F, L, S] of 12-slot rows onto grids 0..10 of every suspension
-// (general kernels for any tile, two passes: 8 and 3 components).
+// (two passes: 8 and 3 components).
 void spread11_launch(pse_ctx *c, const void *vin12, cudaStream_t s) {
   WaveArgs a = wave_args(c);
+  c->nlaunch += 2;
+  if (c->n_cubic == c->nsys) return spread_col11_launch(c, a, vin12, s);
   if (c->prec == PSE_MIXED) {
     spread_p<float, 8, 0, 12, 0>(c, a, vin12, s);
     spread_p<float, 3, 8, 12, 8>(c, a, vin12, s);
@@ -236,7 +238,6 @@ void spread11_launch(pse_ctx *c, const void *vin12, cudaStream_t s) {
     spread_p<double, 8, 0, 12, 0>(c, a, vin12, s);
     spread_p<double, 3, 8, 12, 8>(c, a, vin12, s);
   }
-  c->nlaunch += 2;
 }
 
 }  // namespace pse
