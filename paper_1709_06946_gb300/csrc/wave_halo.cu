@@ -12,33 +12,49 @@
 // shuffles, so every output row is written by one lane with no atomic addition
 // (the tile-owned kernel splits a support over up to 8 tiles and adds the parts).
 // Against the general kernel on 12^3 tiles at N_g = 36: 5 components 55 -> 7.4 us, 8
-// components 39 -> 8.7; the 11-moment product's at N_g = 128 187 -> 124 and 133 -> 60 us.
+// components 39 -> 8.7; the 11-moment product's at N_g = 128 187 -> 105 and 133 -> 60 us.
 // Two CTAs share an SM (about 83 KB each for 5 components, P = 6), so one CTA's
-// staging overlaps the other's read-out.
+// staging overlaps the other's read-out; with enough tiles an item is a whole tile whose
+// planes pass through a ring (halo_layers).
+//
+// Bound by L1: two thirds of the shared-memory and copy wavefronts of the one-layer form
+// are staging (8 per 32 four-byte copies; 3969 points for 64 particles), the rest the
+// read-out's 16-byte reads.  Lanes over 4 components x 8 points (conflict-free stores)
+// made the copies slower (574 -> 1411 us at 2^20), 16 lanes per particle the read-out
+// (540 -> 600).
 #include "wave_common.cuh"
 
 namespace pse {
 namespace {
 
-constexpr int HALO_THREADS = 512;
+// One layer per work item: 512 threads, two CTAs per SM.  Several layers per item: 1024 threads
+// and a ring of planes, one CTA per SM.
+constexpr int HALO_THREADS = 512, RING_THREADS = 1024;
 
 // 4 bytes from global to shared memory without a register round trip (cp.async,
-// cached in L1); completion is awaited with cp_async_wait_all before a barrier.
+// cached in L1); completion is awaited with cp_async_wait before a barrier.
 __device__ __forceinline__ void cp_async4(float *smem, const float *gmem) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// Waits until at most `n` of the thread's latest groups are in flight.
+template <int n>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(n) : "memory");
+}
 constexpr float HALO_LOG2E = 1.4426950408889634f;  // log2(e): exp(-x) = exp2(-x log2 e)
 constexpr int LAYER = CUBE / SUB_SIDE;  // planes of support starts per work item
 
-template <int P> struct Halo {
+template <int P, bool RING = false> struct Halo {
   static constexpr int R = CUBE + P - 1;           // region side along x and y
   static constexpr int RZ = LAYER + P - 1;         // region depth along z
+  static constexpr int NZ = RING ? RZ + LAYER : RZ;  // planes held: a layer's region, and the next layer's new planes
   static constexpr int RX = tile_rx(R, P);         // padded row (RX = P mod 8: conflict-free quarter reads)
   static constexpr int ZS = R * RX;                // plane stride (points)
-  static constexpr int NPT = RZ * ZS;              // points of the staged region
-  static constexpr int NCOL = (P * P + 7) / 8;     // column passes per lane
+  static constexpr int NPT = NZ * ZS;              // points of the staged planes
+  static constexpr int LP = 8;                      // lanes of a particle
+  static constexpr int NCOL = (P * P + LP - 1) / LP;  // column passes per lane
 };
 
 // DEF: deformed lattice with z orthogonal to the sheared plane (as the
@@ -46,148 +62,210 @@ template <int P> struct Halo {
 // exponential of the x-y quadratic form; the z weights use G_zz.
 // COMP0: first grid component read (grid components COMP0 .. COMP0 + C - 1 go
 // to output slots SLOT0 .. SLOT0 + C - 1).  ROW: slots per particle row of vout.
-template <int C, int SLOT0, int P, bool DEF = false, int COMP0 = 0, int ROW = 8>
-__global__ void __launch_bounds__(HALO_THREADS, 2)
-    k_interp_halo(WaveArgs wa, int *queue, const int4 *__restrict__ sp_i0, const float4 *__restrict__ sp_d0,
+//
+// RING: an item is `nl` consecutive layers of a tile.  The planes stay in a ring of
+// slots, so a layer stages only the planes that the one below it did not have (21
+// planes for the four layers of a 16^3 tile at P = 6, not 36), and they are copied while
+// the layer below is read out.
+template <int C, int SLOT0, int P, bool DEF, int COMP0, int ROW, bool RING>
+__global__ void __launch_bounds__(RING ? RING_THREADS : HALO_THREADS, RING ? 1 : 2)
+    k_interp_halo(WaveArgs wa, int *queue, int nl, const int4 *__restrict__ sp_i0, const float4 *__restrict__ sp_d0,
                   const int *__restrict__ fine_start, const float *__restrict__ grid_all, float *__restrict__ vout) {
-  using H = Halo<P>;
-  constexpr int R = H::R, RZ = H::RZ, RX = H::RX, ZS = H::ZS;
+  using H = Halo<P, RING>;
+  constexpr int R = H::R, NZ = H::NZ, RX = H::RX, ZS = H::ZS, LP = H::LP, NT = RING ? RING_THREADS : HALO_THREADS;
   extern __shared__ __align__(32) unsigned char smem_raw[];
   TileL<float, C> tl;
   tl.init(smem_raw, H::NPT);
-  const int lane = threadIdx.x & 31, quarter = lane >> 3, sub = lane & 7, warp = threadIdx.x >> 5;
-  for_each_item(queue, wa.ntiles * SUB_SIDE, [&](int item) {
-    const int tile = item / SUB_SIDE, kz = item % SUB_SIDE;
+  const int lane = threadIdx.x & 31, group = lane / LP, sub = lane % LP, warp = threadIdx.x >> 5;
+  const int per_tile = RING ? (SUB_SIDE + nl - 1) / nl : SUB_SIDE;
+  for_each_item(queue, wa.ntiles * per_tile, [&](int item) {
+    const int tile = item / per_tile, kz0 = (item % per_tile) * (RING ? nl : 1);
+    const int kz1 = RING ? min(kz0 + nl, SUB_SIDE) : kz0 + 1;
     const int si = find_sys(wa.tile0, wa.nsys, tile);
     const SysDev &a = wa.sys[si];
     if (wave_skip(wa, si, a)) return;
     const int Ng = a.Ng;
     int t[3], t0[3];
     tile_of(a, tile - a.tile0, t, t0);
-    const int64_t fb = (int64_t)tile * SUB_BLOCKS + kz * SUB_SIDE * SUB_SIDE;
-    const int beg = fine_start[fb], end = fine_start[fb + SUB_SIDE * SUB_SIDE];
-    if (beg == end) return;
-    // planes [zb, ze) of the tile: those whose sub-block layer 4 z / T is kz
-    const int zb = (kz * a.T[2] + SUB_SIDE - 1) / SUB_SIDE, ze = ((kz + 1) * a.T[2] + SUB_SIDE - 1) / SUB_SIDE;
-    const int z0 = t0[2] + zb, rz = min(ze, tile_width(a, t[2], 2)) - zb + P - 1;
+    const int *fs = fine_start + (int64_t)tile * SUB_BLOCKS;
+    constexpr int LB = SUB_SIDE * SUB_SIDE;  // sub-blocks of a layer
+    if (fs[kz0 * LB] == fs[kz1 * LB]) return;
+    // layer kz holds the planes [first(kz), first(kz + 1)) of the tile: 4 z / T = kz
+    const int wz = tile_width(a, t[2], 2);
+    auto first = [&](int kz) { return min((kz * a.T[2] + SUB_SIDE - 1) / SUB_SIDE, wz); };
     const int rx = tile_width(a, t[0], 0) + P - 1, ry = tile_width(a, t[1], 1) + P - 1;
-    const float *grid = grid_all + a.grid0;
-    // stage the region with asynchronous 4-byte copies straight into the tile layout
-    // (no register round trip: every copy of the thread is in flight before the wait)
-    constexpr int NREG = RZ * R * R;
-    for (int q = threadIdx.x; q < NREG; q += HALO_THREADS) {
-      const int x = q % R, y = (q / R) % R, z = q / (R * R);
-      if (x >= rx || y >= ry || z >= rz) continue;  // a tile of fewer than 16 points
-      int gx = t0[0] + x, gy = t0[1] + y, gz = z0 + z;
-      gx -= gx >= Ng ? Ng : 0;
-      gy -= gy >= Ng ? Ng : 0;
-      gz -= gz >= Ng ? Ng : 0;
-      const size_t g = ((size_t)gz * Ng + gy) * Ng + gx;
-      const int d = z * ZS + y * RX + x;
+    const float *grid = grid_all + a.grid0 + COMP0 * a.gstride;
+    const bool whole = rx == R && ry == R;
+    // planes [za, zb) (from the tile's origin, periodic) into the tile layout; plane z lies in
+    // slot z mod NZ: asynchronous 4-byte copies (no register round trip), or for 5 components
+    // and one layer per item loads and vector stores, U points per thread in flight
+    auto stage = [&](int za, int zb) {
+      constexpr bool REGS = C == 5 && !RING;
+      constexpr int U = REGS ? 2 : 1;
+      const int n = (zb - za) * R * R;
+      for (int q0 = threadIdx.x; q0 < n; q0 += U * NT) {
+        float v[U][C];
+        int d[U];
 #pragma unroll
-      for (int c = 0; c < C; ++c) cp_async4(tl.comp(d, c), grid + (COMP0 + c) * a.gstride + g);
-    }
-    cp_async_wait_all();
+        for (int u = 0; u < U; ++u) {
+          const int q = q0 + u * NT, x = q % R, y = (q / R) % R, dz = q / (R * R), z = za + dz;
+          const bool in = q < n && (whole || (x < rx && y < ry));  // a tile of fewer than 16 points
+          d[u] = in ? (RING ? z % NZ : dz) * ZS + y * RX + x : -1;
+          int gx = t0[0] + x, gy = t0[1] + y, gz = t0[2] + z;
+          gx -= gx >= Ng ? Ng : 0;
+          gy -= gy >= Ng ? Ng : 0;
+          gz -= gz >= Ng ? Ng : 0;
+          const float *g = grid + ((size_t)gz * Ng + gy) * Ng + gx;
+          if (in) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+              if (REGS) v[u][c] = __ldg(g + c * a.gstride);
+              else cp_async4(tl.comp(d[u], c), g + c * a.gstride);
+            }
+          }
+        }
+        if (REGS) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (d[u] >= 0) tl.store(d[u], v[u]);
+        }
+      }
+      cp_async_commit();
+    };
     const float nal = -(float)a.alpha * HALO_LOG2E, hs = (float)a.h, pref = (float)a.pref;
     const float kxx = DEF ? -(float)a.qa[0] * HALO_LOG2E : nal, kyy = DEF ? -(float)a.qa[1] * HALO_LOG2E : nal;
     const float kxy = DEF ? -(float)a.qa[3] * HALO_LOG2E : 0.f, kzz = DEF ? -(float)a.qa[2] * HALO_LOG2E : nal;
-    __syncthreads();  // region staged
-    // four particles per warp per round, one per quarter (warp-uniform loop: the
-    // shuffles below run on all 32 lanes)
-    for (int base = beg + 4 * warp; base < end; base += 4 * (HALO_THREADS / 32)) {
-      const int k = base + quarter;
-      const bool live = k < end;
-      const int ke = live ? k : end - 1;
-      const int4 i0 = sp_i0[ke];
-      const float4 d0 = sp_d0[ke];
-      const int ex = i0.x - t0[0], ey = i0.y - t0[1], ez = i0.z - z0;  // in [0, 16) and [0, LAYER)
-      // 1D weights: lane sub < P holds the x, y and z weights of point sub (P <= 8,
-      // the lanes of a quarter); a larger support has every lane form its own
-      float wz[P], wx = 0.f, wy = 0.f;
-      if constexpr (P <= 8) {
-        const float fs = (float)(sub < P ? sub : 0) * hs;
-        const float ox = d0.x + fs, oy = d0.y + fs, oz = d0.z + fs;
-        wx = exp2f(nal * ox * ox);
-        wy = exp2f(nal * oy * oy);
-        const float wzl = exp2f(kzz * oz * oz);
-#pragma unroll
-        for (int j = 0; j < P; ++j) wz[j] = __shfl_sync(0xffffffffu, wzl, j, 8);
+    stage(first(kz0), first(kz0 + 1) + P - 1);
+    for (int kz = kz0; kz < kz1; ++kz) {
+      const int zl = first(kz);
+      if (RING && kz + 1 < kz1) {
+        stage(first(kz + 1) + P - 1, first(kz + 2) + P - 1);
+        cp_async_wait<1>();
       } else {
-#pragma unroll
-        for (int j = 0; j < P; ++j) {
-          const float oz = d0.z + (float)j * hs;
-          wz[j] = exp2f(kzz * oz * oz);
-        }
+        cp_async_wait<0>();
       }
-      float acc[C];
+      __syncthreads();  // the layer's planes are staged
+      const int beg = fs[kz * LB], end = fs[(kz + 1) * LB];
+      // 32 / LP particles per warp per round (warp-uniform loop: the shuffles below run on
+      // all 32 lanes)
+      for (int base = beg + (32 / LP) * warp; base < end; base += NT / LP) {
+        const int k = base + group;
+        const bool live = k < end;
+        const int ke = live ? k : end - 1;
+        const int4 i0 = sp_i0[ke];
+        const float4 d0 = sp_d0[ke];
+        const int ex = i0.x - t0[0], ey = i0.y - t0[1], ez = i0.z - t0[2];  // in [0, 16), ez in the layer
+        // 1D weights: lane sub < P holds the x, y and z weights of point sub (P <= 8,
+        // the first lanes of a particle); a larger support has every lane form its own
+        float wz[P], wx = 0.f, wy = 0.f;
+        if constexpr (P <= 8) {
+          const float f = (float)(sub < P ? sub : 0) * hs;
+          const float ox = d0.x + f, oy = d0.y + f, oz = d0.z + f;
+          wx = exp2f(nal * ox * ox);
+          wy = exp2f(nal * oy * oy);
+          const float wzl = exp2f(kzz * oz * oz);
 #pragma unroll
-      for (int c = 0; c < C; ++c) acc[c] = 0.f;
-      const int pb = ez * ZS + ey * RX + ex;
-      constexpr int CU = P >= 8 ? 2 : H::NCOL;  // P = 8: partial unroll (register pressure)
-#pragma unroll CU
-      for (int s = 0; s < H::NCOL; ++s) {
-        // this lane's column (px, py) = (c mod P, c / P) of the support, c = sub + 8 s
-        const int cc = sub + 8 * s, px = cc % P, py = cc < P * P ? cc / P : 0;
-        float wxy;
-        if (DEF || P > 8) {  // the column's own x-y weight
-          const float cx = d0.x + (float)px * hs, cy = d0.y + (float)py * hs;
-          wxy = exp2f(kxx * cx * cx + kxy * cx * cy + kyy * cy * cy);
+          for (int j = 0; j < P; ++j) wz[j] = __shfl_sync(0xffffffffu, wzl, j, LP);
         } else {
-          wxy = __shfl_sync(0xffffffffu, wx, px, 8) * __shfl_sync(0xffffffffu, wy, py, 8);
-        }
-        if (cc < P * P) {
-          const int col = pb + py * RX + px;
 #pragma unroll
-          for (int jz = 0; jz < P; ++jz) {
-            float vv[C];
-            tl.load(col + jz * ZS, vv);
-            const float w = wxy * wz[jz];
-#pragma unroll
-            for (int c = 0; c < C; ++c) acc[c] = fmaf(w, vv[c], acc[c]);
+          for (int j = 0; j < P; ++j) {
+            const float oz = d0.z + (float)j * hs;
+            wz[j] = exp2f(kzz * oz * oz);
           }
         }
+        float acc[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[c] = 0.f;
+        const int s0 = RING ? ez % NZ : ez - zl, pb = ey * RX + ex;  // slot of the support's first plane
+        constexpr int CU = P >= 8 ? 2 : H::NCOL;  // P = 8: partial unroll (register pressure)
+#pragma unroll CU
+        for (int s = 0; s < H::NCOL; ++s) {
+          // this lane's column (px, py) = (c mod P, c / P) of the support, c = sub + LP s
+          const int cc = sub + LP * s, px = cc % P, py = cc < P * P ? cc / P : 0;
+          float wxy;
+          if (DEF || P > 8) {  // the column's own x-y weight
+            const float cx = d0.x + (float)px * hs, cy = d0.y + (float)py * hs;
+            wxy = exp2f(kxx * cx * cx + kxy * cx * cy + kyy * cy * cy);
+          } else {
+            wxy = __shfl_sync(0xffffffffu, wx, px, LP) * __shfl_sync(0xffffffffu, wy, py, LP);
+          }
+          if (cc < P * P) {
+            const int col = pb + py * RX + px;
+#pragma unroll
+            for (int jz = 0; jz < P; ++jz) {
+              int sl = s0 + jz;
+              if (RING) sl -= sl >= NZ ? NZ : 0;
+              float vv[C];
+              tl.load(col + sl * ZS, vv);
+              const float w = wxy * wz[jz];
+#pragma unroll
+              for (int c = 0; c < C; ++c) acc[c] = fmaf(w, vv[c], acc[c]);
+            }
+          }
+        }
+#pragma unroll
+        for (int o = LP / 2; o > 0; o >>= 1)
+#pragma unroll
+          for (int c = 0; c < C; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+        // lane c of the particle adds component c
+        float mine = acc[0];
+#pragma unroll
+        for (int c = 1; c < C; ++c) mine = sub == c ? acc[c] : mine;
+        if (live && sub < C) {
+          float *o = vout + ROW * (size_t)k + SLOT0 + sub;
+          *o += pref * mine;
+        }
       }
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-        for (int c = 0; c < C; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-      // lane c of the quarter adds component c
-      float mine = acc[0];
-#pragma unroll
-      for (int c = 1; c < C; ++c) mine = sub == c ? acc[c] : mine;
-      if (live && sub < C) {
-        float *o = vout + ROW * (size_t)k + SLOT0 + sub;
-        *o += pref * mine;
-      }
+      __syncthreads();  // the planes are no longer read when the next ones overwrite them
     }
-    __syncthreads();  // the region is no longer read when the next item overwrites it
   });
 }
 
 // Staged bytes of C components with support P; a CTA may take 223 KB.
-template <int C, int P>
+template <int C, int P, bool RING>
 constexpr size_t halo_bytes() {
-  return (size_t)Halo<P>::NPT * (16 + (C == 5 ? 4 : (C == 8 ? 16 : 0)));
+  return (size_t)Halo<P, RING>::NPT * (16 + (C == 5 ? 4 : (C == 8 ? 16 : 0)));
 }
 
-template <int C, int SLOT0, int P, bool DEF = false, int COMP0 = 0, int ROW = 8>
+template <int C, int SLOT0, int P, bool DEF, int COMP0, int ROW, bool RING>
+void launch_interp_halo_k(pse_ctx *c, const WaveArgs &a, void *vout, int nl, cudaStream_t s) {
+  constexpr int NT = RING ? RING_THREADS : HALO_THREADS;
+  static_assert(halo_bytes<C, P, RING>() <= 223 * 1024, "staged planes");
+  static std::once_flag once;
+  static OccCache occ;
+  const size_t sm = TileL<float, C>::bytes((size_t)Halo<P, RING>::NPT);
+  auto kern = k_interp_halo<C, SLOT0, P, DEF, COMP0, ROW, RING>;
+  set_smem(kern, once);
+  const unsigned grid = wave_grid(c, kern, sm, a.ntiles * (int)ceil_div(SUB_SIDE, nl), occ, NT);
+  int *q = next_queue(c);
+  kern<<<grid, NT, sm, s>>>(a, q, nl, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, c->d_fine_start,
+                            (const float *)c->d_grid, (float *)vout);
+}
+
+// Layers per item: the ring of a whole tile where there are enough tiles per SM.  Measured
+// (us, one layer / ring; 2^20 = 4096 tiles, P = 6 unless said): 8 components 126 / 105 at
+// 512 tiles, 1002 / 722 at 4096; 5 components 68 / 79 at 512, 115 / 109 at 729, 198 / 141 at
+// 729 and P = 8, 549 / 540 at 4096; 3 components 420 / 467 at 4096 (never).  A layer of a
+// ring holds about 64 particles for 128 places, so the ring gains where staging is most
+// of the work (8 components; large supports).  Two layers per item lay between.
+template <int C>
+inline int halo_layers(const pse_ctx *c, const WaveArgs &a) {
+  return a.ntiles >= (C == 8 ? 2 : 4) * c->nsm ? SUB_SIDE : 1;
+}
+
+template <int C, int SLOT0, int P, bool DEF, int COMP0, int ROW>
 void launch_interp_halo(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) {
-  if constexpr (C == 8 && halo_bytes<C, P>() > 223 * 1024) {
+  if constexpr (C == 8 && halo_bytes<C, P, false>() > 223 * 1024) {
     // the staged region of all components does not fit: components 0-4 and 5-7 in two passes
     launch_interp_halo<5, SLOT0, P, DEF, COMP0, ROW>(c, a, vout, s);
     launch_interp_halo<3, SLOT0 + 5, P, DEF, COMP0 + 5, ROW>(c, a, vout, s);
     c->nlaunch += 1;
   } else {
-    static_assert(halo_bytes<C, P>() <= 223 * 1024, "staged region");
-    static std::once_flag once;
-    static OccCache occ;
-    const size_t sm = TileL<float, C>::bytes((size_t)Halo<P>::NPT);
-    auto kern = k_interp_halo<C, SLOT0, P, DEF, COMP0, ROW>;
-    set_smem(kern, once);
-    const unsigned grid = wave_grid(c, kern, sm, a.ntiles * SUB_SIDE, occ, HALO_THREADS);
-    int *q = next_queue(c);
-    kern<<<grid, HALO_THREADS, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, c->d_fine_start,
-                                        (const float *)c->d_grid, (float *)vout);
+    if constexpr (C != 3 && halo_bytes<C, P, true>() <= 223 * 1024) {
+      const int nl = halo_layers<C>(c, a);
+      if (nl > 1) return launch_interp_halo_k<C, SLOT0, P, DEF, COMP0, ROW, true>(c, a, vout, nl, s);
+    }
+    launch_interp_halo_k<C, SLOT0, P, DEF, COMP0, ROW, false>(c, a, vout, 1, s);
   }
 }
 

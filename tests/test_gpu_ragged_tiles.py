@@ -63,6 +63,19 @@ def test_products(pkg, Ng, P, T):
         assert np.linalg.norm(got - ref) < TOL * np.linalg.norm(ref), want
 
 
+# enough tiles for the ring of planes (8 components from two tiles per SM, 5 from four)
+@pytest.mark.parametrize('Ng,P,T,N', [(112, 6, 16, 30000), (130, 5, 15, 30000), (130, 6, 15, 900), (130, 8, 15, 30000),
+                                      (130, 10, 15, 5000)])
+def test_ring_of_planes(pkg, Ng, P, T, N):
+    L = 0.9 * Ng
+    pos, F, _, S = _inputs(N, L)
+    for f, want in ((F, ('U', 'E')), (None, ('E',))):
+        ref, _ = _wave(pkg, pos, f, S, 'fp64', want, L, Ng, P)
+        got, info = _wave(pkg, pos, f, S, 'mixed', want, L, Ng, P)
+        assert info['tile_kernels'] == 1 and info['tile'] == (T, T, T)
+        assert np.linalg.norm(got - ref) < TOL * np.linalg.norm(ref), want
+
+
 @pytest.mark.parametrize('Ng,tile', [(36, (12, 12, 12)), (54, (9, 9, 9)), (32, (8, 16, 16))])
 def test_fixed_tiles_take_the_general_kernels(pkg, Ng, tile):
     L = 0.9 * Ng
