@@ -98,8 +98,8 @@ cudaEvent_t prof_event(pse_ctx *c) {
   return e;
 }
 
-pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s, bool gathered) {
-  if (parts & PSE_PART_REAL) PSE_TRY(real_apply(c, vin, vout, mode, s, gathered));
+pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s) {
+  if (parts & PSE_PART_REAL) PSE_TRY(real_apply(c, vin, vout, mode, s));
   if (parts & PSE_PART_WAVE) PSE_TRY(wave_apply(c, vin, vout, mode, (parts & PSE_PART_REAL) != 0, s));
   if (!(parts & PSE_PART_ALL)) PSE_CUDA_TRY(c, cudaMemsetAsync(vout, 0, c->ts * 8 * (size_t)c->p.N, s));
   return PSE_OK;
@@ -126,29 +126,50 @@ namespace {
 
 pse_status set_all_active(pse_ctx *c, cudaStream_t s) {
   std::fill(c->h_active.begin(), c->h_active.end(), 1);
+  if (c->act_ones) return PSE_OK;  // as the last call left them
   kd_all_active(c, s);
+  c->act_ones = true;
   PSE_CUDA_TRY(c, cudaGetLastError());
   return PSE_OK;
 }
 
-// Runs `body` (one Krylov iteration, launched on the stream it is given, with the loop's
-// condition handle inside a capture) until
-// the control kernels clear the loop flag, at most `cap` times.  Outside a
-// capture this is a host loop that reads the flag (and the active set) after
-// every iteration; while the step is being captured it becomes a conditional
-// while node whose body graph is captured from a second stream, so the whole
-// loop runs on the device.
-template <typename Body>
-pse_status krylov_loop(pse_ctx *c, int cap, cudaStream_t s, Body &&body) {
+// Runs Krylov iterations until the control kernels clear the loop flag, at most `cap`
+// times.  An iteration is first(t) (kernels that pass over converged suspensions: with
+// none left they end at once), second(t) and step(t, h, graph) (the vector and control
+// kernels).
+//
+// Outside a capture this is a host loop that reads the flag and the active set of every
+// iteration, and queues the next iteration's first part (all of it, when there is no
+// second part) before it waits for them, so the device does not idle while the host
+// wakes up and launches: 42 us per iteration for a sample of 50000 particles, 50 for a
+// step of 30000.  While the step is being captured it becomes a conditional while node
+// whose body graph is captured from a second stream, so the whole loop runs on the
+// device.
+template <typename First, typename Second, typename Step>
+pse_status krylov_loop(pse_ctx *c, int cap, bool has_second, cudaStream_t s, First &&first, Second &&second,
+                       Step &&step) {
   if (!c->capturing) {
-    for (int j = 0; j < cap; ++j) {
-      PSE_TRY(body(s, 0, 0));
+    const size_t nf = 1 + (size_t)c->nsys;
+    auto rest = [&](int j) -> pse_status {  // everything behind first() of iteration j, and its flags
+      if (has_second) PSE_TRY(second(s));
+      PSE_TRY(step(s, 0, 0));
       // the flag and, right behind it, the active set
-      PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_flag, c->kd.flag, sizeof(int) * (1 + c->nsys), cudaMemcpyDeviceToHost, s));
-      PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
+      PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_flag + (j & 1) * nf, c->kd.flag, sizeof(int) * nf, cudaMemcpyDeviceToHost, s));
+      PSE_CUDA_TRY(c, cudaEventRecord(c->flag_ev[j & 1], s));
+      return PSE_OK;
+    };
+    PSE_TRY(first(s));
+    PSE_TRY(rest(0));
+    for (int j = 0; j < cap; ++j) {
+      const bool more = j + 1 < cap;
+      if (more) PSE_TRY(first(s));
+      if (more && !has_second) PSE_TRY(rest(j + 1));
+      PSE_CUDA_TRY(c, cudaEventSynchronize(c->flag_ev[j & 1]));
       c->h2d_pending = false;
-      std::copy(c->h_flag + 1, c->h_flag + 1 + c->nsys, c->h_active.begin());
-      if (!c->h_flag[0]) break;
+      const int *f = c->h_flag + (j & 1) * nf;
+      std::copy(f + 1, f + nf, c->h_active.begin());
+      if (!f[0]) break;
+      if (more && has_second) PSE_TRY(rest(j + 1));
     }
     return PSE_OK;
   }
@@ -180,7 +201,9 @@ pse_status krylov_loop(pse_ctx *c, int cap, cudaStream_t s, Body &&body) {
   cudaGraph_t body_g = np.conditional.phGraph_out[0];
   PSE_CUDA_TRY(c, cudaStreamBeginCaptureToGraph(c->cap_stream, body_g, nullptr, nullptr, 0,
                                                 cudaStreamCaptureModeRelaxed));
-  pse_status st = body(c->cap_stream, h, 1);
+  pse_status st = first(c->cap_stream);
+  if (st == PSE_OK && has_second) st = second(c->cap_stream);
+  if (st == PSE_OK) st = step(c->cap_stream, h, 1);
   cudaGraph_t out_g = nullptr;
   cudaError_t e = cudaStreamEndCapture(c->cap_stream, &out_g);
   PSE_TRY(st);
@@ -188,37 +211,38 @@ pse_status krylov_loop(pse_ctx *c, int cap, cudaStream_t s, Body &&body) {
   return PSE_OK;
 }
 
-// One recurrence from z (Lanczos) or b (GMRES) in the order of its basis rows; `apply`
-// launches w = A d_vin on the given stream.
-template <typename Apply>
-pse_status krylov(pse_ctx *c, const void *z, void *w, bool gm, int cap, cudaStream_t s, Apply &&apply) {
+// One recurrence from z (Lanczos: w = M_r v, GMRES: w = M_ES v) in the order of its basis rows.
+pse_status krylov(pse_ctx *c, const void *z, void *w, bool gm, int cap, cudaStream_t s) {
   std::fill(c->h_active.begin(), c->h_active.end(), 1);
+  c->act_ones = false;
   PSE_TRY(kr_start(c, z, gm, s));
   PSE_TRY(kr_next(c, z, s));
-  PSE_TRY(krylov_loop(c, cap, s, [&](cudaStream_t t, cudaGraphConditionalHandle h, int graph) {
-    PSE_TRY(apply(t));
-    PSE_TRY(kr_step(c, w, gm, cap, h, graph, t));
-    return kr_next(c, w, t);
-  }));
+  PSE_TRY(krylov_loop(
+      c, cap, gm, s,
+      [&](cudaStream_t t) {
+        PSE_TRY(real_apply(c, c->d_vin, w, gm ? M_SE : M_FULL, t, true));
+        return gm ? wave_spread(c, c->d_vin, M_SE, t) : PSE_OK;
+      },
+      [&](cudaStream_t t) { return wave_finish(c, w, M_SE, t); },
+      [&](cudaStream_t t, cudaGraphConditionalHandle h, int graph) {
+        PSE_TRY(kr_step(c, w, gm, cap, h, graph, t));
+        return kr_next(c, w, t);
+      }));
   return set_all_active(c, s);
 }
 
 // y = M_r^{1/2} z by Lanczos with full reorthogonalisation (Sec. 3.2), per
 // suspension, stopping rule and tridiagonal square root on the device.
 pse_status lanczos(pse_ctx *c, const void *z, void *y, void *w, cudaStream_t s) {
-  const int cap = c->lanczos_max;
-  PSE_TRY(krylov(c, z, w, false, cap, s,
-                 [&](cudaStream_t t) { return real_apply(c, c->d_vin, w, M_FULL, t, true); }));
-  return combine_set(c, y, c->d_basis, c->d_nrows, cap, CO_Y, s);
+  PSE_TRY(krylov(c, z, w, false, c->lanczos_max, s));
+  return combine_set(c, y, c->d_basis, c->d_nrows, c->lanczos_max, CO_Y, s);
 }
 
 // Unrestarted GMRES (x0 = 0) for M_ES x = b at the current configuration, per
 // suspension; stops at |r|/|b| <= tol.  b and x hold the stresslet in slots 3..7.
 pse_status gmres(pse_ctx *c, const void *b, void *x, void *w, cudaStream_t s) {
-  const int cap = c->krylov_max;
-  PSE_TRY(krylov(c, b, w, true, cap, s,
-                 [&](cudaStream_t t) { return mobility(c, c->d_vin, w, M_SE, PSE_PART_ALL, t, true); }));
-  return combine_set(c, x, c->d_basis, c->d_nrows, cap, CO_Y, s);
+  PSE_TRY(krylov(c, b, w, true, c->krylov_max, s));
+  return combine_set(c, x, c->d_basis, c->d_nrows, c->krylov_max, CO_Y, s);
 }
 
 // Unscaled Brownian slip [M_r^{1/2} w1 + M_w^{1/2} dW2] in sorted order into out.
@@ -244,19 +268,22 @@ pse_status check_inputs(pse_ctx *c, const void *p, int64_t n, bool dbl, cudaStre
   return PSE_OK;
 }
 
-// Per-suspension iteration counts and residuals of the last Lanczos / GMRES run
-// (read from the device after the stream has been synchronised); returns
+size_t stats_bytes(const pse_ctx *c) { return (2 * sizeof(double) + 4 * sizeof(int)) * (size_t)c->nsys; }
+
+// Queues a copy of the Krylov statistics as they stand on the stream into host slot `slot`.
+pse_status queue_krylov_stats(pse_ctx *c, int slot, cudaStream_t s) {
+  PSE_CUDA_TRY(c, cudaMemcpyAsync((char *)c->h_stats + slot * stats_bytes(c), c->kd.stats, stats_bytes(c),
+                                  cudaMemcpyDeviceToHost, s));
+  return PSE_OK;
+}
+
+// Per-suspension iteration counts and residuals of the Lanczos / GMRES run whose
+// statistics are in a host slot (after the stream has been synchronised); returns
 // NOT_CONVERGED if a cap was reached.
-pse_status read_krylov_stats(pse_ctx *c, bool lz, bool gm, cudaStream_t s) {
+pse_status take_krylov_stats(pse_ctx *c, int slot, bool lz, bool gm) {
   const int ns = c->nsys;
-  std::vector<int> it(2 * ns);
-  std::vector<double> r(2 * ns);
-  PSE_CUDA_TRY(c, cudaMemcpyAsync(it.data(), c->kd.l_it, sizeof(int) * 2 * ns, cudaMemcpyDeviceToHost, s));
-  PSE_CUDA_TRY(c, cudaMemcpyAsync(r.data(), c->kd.l_err, sizeof(double) * ns, cudaMemcpyDeviceToHost, s));
-  PSE_CUDA_TRY(c, cudaMemcpyAsync(r.data() + ns, c->kd.g_rel, sizeof(double) * ns, cudaMemcpyDeviceToHost, s));
-  std::vector<int> gi(2 * ns);
-  PSE_CUDA_TRY(c, cudaMemcpyAsync(gi.data(), c->kd.g_it, sizeof(int) * 2 * ns, cudaMemcpyDeviceToHost, s));
-  PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
+  const double *r = (const double *)((const char *)c->h_stats + slot * stats_bytes(c));
+  const int *it = (const int *)(r + 2 * ns), *gi = it + 2 * ns;
   bool capped = false;
   for (int q = 0; q < ns; ++q) {
     pse_stats &o = c->sys_stats[q];
@@ -301,8 +328,6 @@ size_t w2_bytes(const pse_ctx *c) { return c->ts * 6 * (size_t)c->nk_tot; }
 pse_status step_body(pse_ctx *c, const void *dFP, double dt, const void *dw1, const void *dw2, uint64_t seed,
                      uint64_t stepno, cudaStream_t s) {
   const Params &p = c->p;
-  const int64_t N = p.N;
-  const size_t vb = c->ts * 8 * N;
   // 1. Brownian slip at x_k (unconstrained), user order, scaled by sqrt(2kT/dt)
   PSE_TRY(setup_config(c, c->d_pos0, s));
   PSE_TRY(sample_sorted(c, dw1, dw2, seed, stepno, c->d_v[2], s));
@@ -310,25 +335,20 @@ pse_status step_body(pse_ctx *c, const void *dFP, double dt, const void *dw1, co
   // 2. x_{k+1/2} = x_k + dt/2 U^B
   PSE_TRY(midpoint(c, c->d_pos0, c->d_B, 0.5 * dt, c->d_posh, s));
   PSE_TRY(setup_config(c, c->d_posh, s));
-  // 3. M_ES S = -E^B - M_EF F^P at x_{k+1/2}
-  PSE_TRY(gather_user8(c, c->d_B, c->d_v[2], s));
-  PSE_TRY(vscale(c, c->d_v[2], c->d_v[2], -1.0, -1, s));
+  // 3. M_ES S = -E^B - M_EF F^P at x_{k+1/2}; the Krylov vectors have no force slots, nor has S
   if (dFP) {
-    PSE_TRY(gather_in(c, dFP, nullptr, c->d_v[3], s));
+    PSE_TRY(gather_in(c, dFP, nullptr, c->d_v[3], false, s));
     PSE_TRY(mobility(c, c->d_v[3], c->d_v[4], M_FULL, PSE_PART_ALL, s));
-    PSE_TRY(combine_sub(c, c->d_v[2], c->d_v[4], 1, CO_ONE, s));
   }
-  PSE_TRY(vzero_slots(c, c->d_v[2], 0, 3, s));
+  PSE_TRY(krylov_rhs(c, c->d_B, true, dFP ? c->d_v[4] : nullptr, c->d_v[2], s));
   PSE_TRY(gmres(c, c->d_v[2], c->d_v[5], c->d_v[1], s));
-  PSE_TRY(vzero_slots(c, c->d_v[5], 0, 3, s));
   // 4. U = U^B + M_UF F^P + M_US S;  x_{k+1} = x_k + dt U
+  const void *fs = c->d_v[5];
   if (dFP) {
-    PSE_TRY(gather_in(c, dFP, nullptr, c->d_v[3], s));
-    PSE_TRY(combine_sub(c, c->d_v[3], c->d_v[5], 1, CO_MONE, s));
-  } else {
-    PSE_CUDA_TRY(c, cudaMemcpyAsync(c->d_v[3], c->d_v[5], vb, cudaMemcpyDeviceToDevice, s));
+    PSE_TRY(gather_join(c, dFP, c->d_v[5], c->d_v[3], s));
+    fs = c->d_v[3];
   }
-  PSE_TRY(mobility(c, c->d_v[3], c->d_v[4], dFP ? M_FSU : M_SU, PSE_PART_ALL, s));
+  PSE_TRY(mobility(c, fs, c->d_v[4], dFP ? M_FSU : M_SU, PSE_PART_ALL, s));
   return final_update(c, c->d_pos0, c->d_B, c->d_v[4], dt, c->d_posout, s);
 }
 
@@ -378,21 +398,17 @@ pse_status capture_step(pse_ctx *c, const void *dFP, double dt) {
   return PSE_OK;
 }
 
-// After a graph step: non-finite inputs, neighbour-list overflow (the list grows
-// and the step is repeated eagerly), per-suspension pair counts.
-pse_status graph_checks(pse_ctx *c, bool *redo, cudaStream_t s) {
+// After a graph step (its status words copied and the stream synchronised): non-finite
+// inputs, neighbour-list overflow (the list grows and the step is repeated eagerly),
+// per-suspension pair counts.
+pse_status graph_checks(pse_ctx *c, bool *redo) {
   const int ns = c->nsys;
-  PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_pinned_int, c->d_flag, sizeof(int) * 4, cudaMemcpyDeviceToHost, s));
-  PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_nbr_tot, c->d_nbr_tot, 2 * sizeof(unsigned long long) * ns,
-                                  cudaMemcpyDeviceToHost, s));
-  PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
-  c->h2d_pending = false;
   *redo = false;
-  if (c->h_pinned_int[0]) {
+  if (c->h_status[0]) {
     c->err = "non-finite particle position";
     return PSE_ERR_NONFINITE;
   }
-  if (c->h_pinned_int[2]) {
+  if (c->h_status[2]) {
     c->err = "non-finite input";
     return PSE_ERR_NONFINITE;
   }
@@ -402,7 +418,7 @@ pse_status graph_checks(pse_ctx *c, bool *redo, cudaStream_t s) {
     c->npairs_sys[q] = (int64_t)c->h_nbr_tot[2 * q];
     c->npairs += c->npairs_sys[q];
   }
-  *redo = c->h_pinned_int[1] != 0;  // a list overflowed in one of the two builds
+  *redo = c->h_status[1] != 0;  // a list overflowed in one of the two builds
   return PSE_OK;
 }
 
@@ -458,27 +474,38 @@ pse_status step_impl(pse_ctx *c, double *pos, const void *FP, double dt, const v
     c->h2d_pending = true;
     PSE_CUDA_TRY(c, cudaGraphLaunch(c->g_exec, s));
     c->nlaunch += 1;
+    // device outputs are written behind the graph, by kernels that write nothing if a
+    // status word is set, so the host waits once
+    PSE_TRY(commit_positions(c, c->d_posout, (double *)dpos, s));
+    if (S_out && is_device_ptr(S_out)) PSE_TRY(scatter_out(c, c->d_v[5], nullptr, S_out, 1.0, s, true));
+    PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_status, c->d_flag, 16 + 2 * sizeof(unsigned long long) * c->nsys,
+                                    cudaMemcpyDeviceToHost, s));
+    PSE_TRY(queue_krylov_stats(c, 0, s));
+    PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
+    c->h2d_pending = false;
     bool redo = false;
-    PSE_TRY(graph_checks(c, &redo, s));
+    PSE_TRY(graph_checks(c, &redo));
     if (redo) ++c->layout_version;  // the eager rerun below grows the lists; recapture next time
     done = !redo;
   }
+  const bool fresh = !done;  // launched from the host: its outputs are still to be written
   if (!done) {
     PSE_TRY(stage(c, 1, FP, c->ts * 3 * N, true, s, &dFP));
     PSE_TRY(check_inputs(c, dFP, 3 * N, c->prec == PSE_FP64, s));
     PSE_TRY(step_body(c, dFP, dt, dw1, dw2, seed, stepno, s));
+    PSE_CUDA_TRY(c, cudaMemcpyAsync(dpos, c->d_posout, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s));
+    PSE_TRY(queue_krylov_stats(c, 0, s));
   }
-  PSE_CUDA_TRY(c, cudaMemcpyAsync(dpos, c->d_posout, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s));
   PSE_TRY(unstage(c, pos, dpos, sizeof(double) * 3 * N, s));
-  if (S_out) {
+  if (S_out && (fresh || !is_device_ptr(S_out))) {
     void *dS;
     PSE_TRY(stage(c, 4, S_out, c->ts * 5 * N, false, s, &dS));
     PSE_TRY(scatter_out(c, c->d_v[5], nullptr, dS, 1.0, s));
     PSE_TRY(unstage(c, S_out, dS, c->ts * 5 * N, s));
   }
-  PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
+  if (fresh || dpos != (void *)pos || (S_out && !is_device_ptr(S_out))) PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
   c->h2d_pending = false;
-  pse_status ks = read_krylov_stats(c, true, true, s);
+  pse_status ks = take_krylov_stats(c, 0, true, true);
   gather_stats(c, st);
   return ks;
 }
@@ -522,45 +549,29 @@ pse_status rfd_impl(pse_ctx *c, double *pos, const void *FP, double dt, double d
   int kit = 0;
   double krel = 0.0;
   bool capped = false;
-  auto solve_stats = [&]() -> pse_status {
-    pse_status ks = read_krylov_stats(c, false, true, s);
-    capped = capped || ks == PSE_ERR_NOT_CONVERGED;
-    for (const pse_stats &q : c->sys_stats) {
-      kit += q.krylov_iters;
-      krel = std::max(krel, q.krylov_relres);
-    }
-    return (ks == PSE_OK || ks == PSE_ERR_NOT_CONVERGED) ? PSE_OK : ks;
-  };
   // 1. at x_k: slip, constrained solve, U = U^B + M_UF F^P + M_US S
   PSE_TRY(setup_config(c, c->d_pos0, s));
   PSE_TRY(sample_sorted(c, dw1, dw2, seed, stepno, c->d_v[2], s));
   PSE_TRY(scatter_user8(c, c->d_v[2], c->d_B, std::sqrt(2.0 * p.kT / dt), s));
-  PSE_TRY(read_krylov_stats(c, true, false, s) == PSE_ERR_CUDA ? PSE_ERR_CUDA : PSE_OK);
-  const pse_stats lz0 = c->sys_stats.empty() ? pse_stats{} : c->sys_stats[0];
-  PSE_TRY(gather_user8(c, c->d_B, c->d_v[2], s));
-  PSE_TRY(vscale(c, c->d_v[2], c->d_v[2], -1.0, -1, s));
   if (dFP) {
-    PSE_TRY(gather_in(c, dFP, nullptr, c->d_v[3], s));
+    PSE_TRY(gather_in(c, dFP, nullptr, c->d_v[3], false, s));
     PSE_TRY(mobility(c, c->d_v[3], c->d_v[4], M_FULL, PSE_PART_ALL, s));
-    PSE_TRY(combine_sub(c, c->d_v[2], c->d_v[4], 1, CO_ONE, s));
   }
-  PSE_TRY(vzero_slots(c, c->d_v[2], 0, 3, s));
+  PSE_TRY(krylov_rhs(c, c->d_B, true, dFP ? c->d_v[4] : nullptr, c->d_v[2], s));
   PSE_TRY(gmres(c, c->d_v[2], c->d_v[5], c->d_v[1], s));
-  PSE_TRY(vzero_slots(c, c->d_v[5], 0, 3, s));
-  PSE_TRY(solve_stats());
+  PSE_TRY(queue_krylov_stats(c, 0, s));
   if (S_out) {
     void *dS;
     PSE_TRY(stage(c, 4, S_out, c->ts * 5 * N, false, s, &dS));
     PSE_TRY(scatter_out(c, c->d_v[5], nullptr, dS, 1.0, s));
     PSE_TRY(unstage(c, S_out, dS, c->ts * 5 * N, s));
   }
+  const void *fs = c->d_v[5];
   if (dFP) {
-    PSE_TRY(gather_in(c, dFP, nullptr, c->d_v[3], s));
-    PSE_TRY(combine_sub(c, c->d_v[3], c->d_v[5], 1, CO_MONE, s));
-  } else {
-    PSE_CUDA_TRY(c, cudaMemcpyAsync(c->d_v[3], c->d_v[5], vb, cudaMemcpyDeviceToDevice, s));
+    PSE_TRY(gather_join(c, dFP, c->d_v[5], c->d_v[3], s));
+    fs = c->d_v[3];
   }
-  PSE_TRY(mobility(c, c->d_v[3], c->d_v[4], dFP ? M_FSU : M_SU, PSE_PART_ALL, s));
+  PSE_TRY(mobility(c, fs, c->d_v[4], dFP ? M_FSU : M_SU, PSE_PART_ALL, s));
   PSE_TRY(scatter_user8(c, c->d_v[4], U0, 1.0, s));
   // 2. R_FU^{-1}(x_k +- delta/2 W) W, one solve each
   PSE_TRY(rfd_noise(c, dwt, seed, stepno, W8, s));
@@ -569,11 +580,9 @@ pse_status rfd_impl(pse_ctx *c, double *pos, const void *FP, double dt, double d
     PSE_TRY(setup_config(c, c->d_posh, s));
     PSE_TRY(gather_user8(c, W8, c->d_v[0], s));
     PSE_TRY(mobility(c, c->d_v[0], c->d_v[3], M_FULL, PSE_PART_ALL, s));  // (M_UF W, M_EF W)
-    PSE_TRY(vscale(c, c->d_v[2], c->d_v[3], -1.0, -1, s));
-    PSE_TRY(vzero_slots(c, c->d_v[2], 0, 3, s));
+    PSE_TRY(krylov_rhs(c, c->d_v[3], false, nullptr, c->d_v[2], s));
     PSE_TRY(gmres(c, c->d_v[2], c->d_v[5], c->d_v[1], s));
-    PSE_TRY(vzero_slots(c, c->d_v[5], 0, 3, s));
-    PSE_TRY(solve_stats());
+    PSE_TRY(queue_krylov_stats(c, 1 + side, s));
     PSE_TRY(mobility(c, c->d_v[5], c->d_v[4], M_SU, PSE_PART_ALL, s));     // M_US S
     PSE_TRY(combine_sub(c, c->d_v[4], c->d_v[3], 1, CO_MONE, s));           // + M_UF W
     PSE_TRY(scatter_user8(c, c->d_v[4], side ? Rm : Rp, 1.0, s));
@@ -584,9 +593,15 @@ pse_status rfd_impl(pse_ctx *c, double *pos, const void *FP, double dt, double d
   PSE_TRY(unstage(c, pos, dpos, sizeof(double) * 3 * N, s));
   PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
   c->h2d_pending = false;
+  take_krylov_stats(c, 0, true, false);  // the Lanczos run's own cap does not fail the step
+  for (int slot = 0; slot < 3; ++slot) {
+    capped = take_krylov_stats(c, slot, false, true) == PSE_ERR_NOT_CONVERGED || capped;
+    for (const pse_stats &q : c->sys_stats) {
+      kit += q.krylov_iters;
+      krel = std::max(krel, q.krylov_relres);
+    }
+  }
   for (pse_stats &q : c->sys_stats) {
-    q.lanczos_iters = lz0.lanczos_iters;
-    q.lanczos_change = lz0.lanczos_change;
     q.krylov_iters = kit;
     q.krylov_relres = krel;
   }
@@ -623,7 +638,7 @@ int64_t estimate_bytes(const pse_ctx *c) {
   int rows = std::max(c->lanczos_max, c->krylov_max) + 1;
   int64_t b = 0;
   b += (int64_t)ts * 8 * 2048 * 16;                 // table (upper bound)
-  b += Nt * (24 + 4 * 6 + 16 + 12 * (int64_t)ts);  // positions, keys, perm/inv, cells, records (two orders)
+  b += Nt * (24 + 4 * 7 + 16 + 12 * (int64_t)ts);  // positions, keys, perm/inv, cells, records (two orders)
   b += nbr * 4 * (int64_t)ts + (Nt + 1) * 4;
   b += (ntile * (8 + 8 * SUB_BLOCKS) + ncell * 8);
   const int64_t ncomp = c->opt.torque ? 11 : 8;
@@ -757,6 +772,21 @@ pse_status choose_group(pse_ctx *c, int nsys, const int64_t *N, const double *L,
   c->lanczos_tol = o.lanczos_tol < 0 ? shared.tol : o.lanczos_tol;
   c->krylov_tol = o.krylov_tol < 0 ? shared.tol : o.krylov_tol;
   return PSE_OK;
+}
+
+// The block of status words, neighbour totals and bin counts (pse_ctx) for ntiles tiles.
+bool alloc_counts(pse_ctx *c, int64_t ntiles) {
+  const size_t head = 16 + 2 * sizeof(unsigned long long) * (size_t)c->nsys, nf = (size_t)ntiles * SUB_BLOCKS + 1;
+  char *b = (char *)dalloc(c, head + sizeof(int) * (nf + (size_t)c->ncells + 1));
+  int *t = (int *)dalloc(c, sizeof(int) * ((size_t)ntiles + 1));
+  if (!b || !t) return false;
+  c->d_flag = (int *)b;
+  c->d_nbr_tot = (unsigned long long *)(b + 16);
+  c->d_fine_start = (int *)(b + head);
+  c->d_cell_start = c->d_fine_start + nf;
+  c->d_tile_start = t;
+  c->tile_cap = ntiles;
+  return true;
 }
 
 pse_status create_group(pse_ctx *c, const pse_options &o) {
@@ -898,12 +928,8 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
   c->d_cell_key = (int *)A(sizeof(int) * N);
   c->d_perm = (int *)A(sizeof(int) * N);
   c->d_inv = (int *)A(sizeof(int) * N);
-  c->d_tile_start = (int *)A(sizeof(int) * (c->ntiles + 1));
-  c->d_tile_cur = (int *)A(sizeof(int) * (c->ntiles + 1));
-  c->d_fine_start = (int *)A(sizeof(int) * (c->ntiles * SUB_BLOCKS + 1));
-  c->d_fine_cur = (int *)A(sizeof(int) * (c->ntiles * SUB_BLOCKS + 1));
-  c->d_cell_start = (int *)A(sizeof(int) * (c->ncells + 1));
-  c->d_cell_cur = (int *)A(sizeof(int) * (c->ncells + 1));
+  c->d_rank = (int *)A(sizeof(int) * N);
+  if (!alloc_counts(c, c->ntiles)) fail = true;
   c->d_cell_list = (int *)A(sizeof(int) * N);
   c->d_vcell = A(8 * ts * (size_t)N);
   if (o.torque) {
@@ -928,16 +954,13 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
     return PSE_ERR_INVALID_ARG;
   }
   c->d_nbr_geo = A(4 * ts * (size_t)c->nbr_cap);
-  c->d_nbr_tot = (unsigned long long *)A(2 * sizeof(unsigned long long) * ns);
   c->d_sp_i0 = A(sizeof(int4) * N);
   c->d_sp_d0 = A(4 * ts * N);
   c->d_rs = A(4 * ts * N);
   c->d_rs_cell = A(4 * ts * N);
   int64_t big = std::max<int64_t>(std::max<int64_t>(c->ntiles * SUB_BLOCKS, c->ncells), N) + 1;
   c->scan_cap = scan_tmp_ints(big);
-  c->tile_cap = c->ntiles;
   c->d_scan_tmp = (int *)A(sizeof(int) * (size_t)c->scan_cap);
-  c->d_flag = (int *)A(sizeof(int) * 4);
   c->d_grid = A(ts * (size_t)c->grid_elems);
   c->d_cgrid = A(2 * ts * (size_t)c->cgrid_elems);
   for (int i = 0; i < 6; ++i) c->d_v[i] = A(ts * 8 * N);
@@ -955,9 +978,12 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
     k.gmax = M;
     k.ltol = c->lanczos_tol;
     k.gtol = c->krylov_tol;
-    k.l_it = (int *)A(sizeof(int) * 2 * ns);   // l_it then l_capped (read back together)
+    k.stats = (double *)A(stats_bytes(c));
+    k.l_err = k.stats;
+    k.g_rel = k.l_err + ns;
+    k.l_it = (int *)(k.g_rel + ns);
     k.l_capped = k.l_it + ns;
-    k.g_it = (int *)A(sizeof(int) * 2 * ns);   // g_it then g_capped
+    k.g_it = k.l_capped + ns;
     k.g_capped = k.g_it + ns;
     k.l_alpha = (double *)A(sizeof(double) * ns * (size_t)L);
     k.l_beta = (double *)A(sizeof(double) * ns * (size_t)L);
@@ -972,13 +998,11 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
     }
     k.l_nodes = nodes;
     k.l_b0 = (double *)A(sizeof(double) * ns);
-    k.l_err = (double *)A(sizeof(double) * ns);
     k.g_H = (double *)A(sizeof(double) * ns * (size_t)(M + 1) * M);
     k.g_cs = (double *)A(sizeof(double) * ns * (size_t)M);
     k.g_sn = (double *)A(sizeof(double) * ns * (size_t)M);
     k.g_g = (double *)A(sizeof(double) * ns * (size_t)(M + 1));
     k.g_beta = (double *)A(sizeof(double) * ns);
-    k.g_rel = (double *)A(sizeof(double) * ns);
   }
   c->d_coef = (double *)A(sizeof(double) * COEF_STRIDE * (size_t)ns);
   c->kd.coef = c->d_coef;
@@ -988,16 +1012,16 @@ pse_status create_group(pse_ctx *c, const pse_options &o) {
     c->err = "device allocation failed (" + std::to_string(c->dev_bytes) + " bytes so far)";
     return PSE_ERR_OOM;
   }
-  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_dots, sizeof(double) * COEF_STRIDE * (size_t)ns));
-  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_wbuf, sizeof(double) * COEF_STRIDE * (size_t)ns));
-  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_pinned_int, sizeof(int) * (8 + 2 * (size_t)ns)));
-  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_nbr_tot, 2 * sizeof(unsigned long long) * ns));
-  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_flag, sizeof(int) * (1 + (size_t)ns)));
+  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_stats, STAT_SLOTS * stats_bytes(c)));
+  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_pinned_int, sizeof(int) * 8));
+  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_status, 16 + 2 * sizeof(unsigned long long) * ns));
+  c->h_nbr_tot = (unsigned long long *)(c->h_status + 4);
+  PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_flag, sizeof(int) * 2 * (1 + (size_t)ns)));
+  for (cudaEvent_t &e : c->flag_ev) PSE_CUDA_TRY(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   PSE_CUDA_TRY(c, cudaMallocHost((void **)&c->h_rng, 2 * sizeof(uint64_t)));
   PSE_CUDA_TRY(c, cudaMemset(c->kd.iter, 0, sizeof(int) * 4));
   PSE_CUDA_TRY(c, cudaMemset(c->d_done, 0, sizeof(int) * ((size_t)ns + 1)));
-  PSE_CUDA_TRY(c, cudaMemset(c->kd.l_it, 0, sizeof(int) * 2 * ns));
-  PSE_CUDA_TRY(c, cudaMemset(c->kd.g_it, 0, sizeof(int) * 2 * ns));
+  PSE_CUDA_TRY(c, cudaMemset(c->kd.stats, 0, stats_bytes(c)));
   PSE_CUDA_TRY(c, cudaMemcpy(c->d_sys, c->hs.data(), sizeof(SysDev) * ns, cudaMemcpyHostToDevice));
   PSE_CUDA_TRY(c, cudaMemcpy(c->d_p0, p0.data(), sizeof(int64_t) * (ns + 1), cudaMemcpyHostToDevice));
   PSE_CUDA_TRY(c, cudaMemcpy(c->d_k0, k0.data(), sizeof(int64_t) * (ns + 1), cudaMemcpyHostToDevice));
@@ -1112,11 +1136,12 @@ void destroy_impl(pse_ctx *c) {
   c->g_exec = nullptr;
   c->g_graph = nullptr;
   c->cap_stream = nullptr;
+  for (cudaEvent_t &e : c->flag_ev)
+    if (e) cudaEventDestroy(e);
   for (void *q : c->allocs) cudaFree(q);
-  if (c->h_dots) cudaFreeHost(c->h_dots);
-  if (c->h_wbuf) cudaFreeHost(c->h_wbuf);
+  if (c->h_stats) cudaFreeHost(c->h_stats);
   if (c->h_pinned_int) cudaFreeHost(c->h_pinned_int);
-  if (c->h_nbr_tot) cudaFreeHost(c->h_nbr_tot);
+  if (c->h_status) cudaFreeHost(c->h_status);
   if (c->h_flag) cudaFreeHost(c->h_flag);
   if (c->h_rng) cudaFreeHost(c->h_rng);
   c->allocs.clear();
@@ -1136,19 +1161,9 @@ pse_status retile(pse_ctx *c, const int caps[3]) {
     tile0[q + 1] = tile0[q] + ps[q].ntile[0] * ps[q].ntile[1] * ps[q].ntile[2];
   }
   const int64_t nt = tile0[c->nsys];
-  if (nt > c->tile_cap) {
-    void *a = dalloc(c, sizeof(int) * (size_t)(nt + 1)), *b = dalloc(c, sizeof(int) * (size_t)(nt + 1));
-    void *fa = dalloc(c, sizeof(int) * (size_t)(nt * SUB_BLOCKS + 1));
-    void *fb = dalloc(c, sizeof(int) * (size_t)(nt * SUB_BLOCKS + 1));
-    if (!a || !b || !fa || !fb) {
-      c->err = "cannot allocate tile arrays";
-      return PSE_ERR_OOM;
-    }
-    c->d_tile_start = (int *)a;
-    c->d_tile_cur = (int *)b;
-    c->d_fine_start = (int *)fa;
-    c->d_fine_cur = (int *)fb;
-    c->tile_cap = nt;
+  if (nt > c->tile_cap && !alloc_counts(c, nt)) {
+    c->err = "cannot allocate tile arrays";
+    return PSE_ERR_OOM;
   }
   int64_t need = scan_tmp_ints(std::max<int64_t>(std::max<int64_t>(nt * SUB_BLOCKS, c->ncells), c->p.N) + 1);
   if (need > c->scan_cap) {
@@ -1495,11 +1510,12 @@ pse_status pse_mobility_apply_parts(pse_handle h, const double *pos, const void 
   PSE_TRY(stage(c, 3, U, c->ts * 3 * N, false, s, &dU));
   PSE_TRY(stage(c, 4, E, c->ts * 5 * N, false, s, &dE));
   PSE_TRY(setup_config(c, (const double *)dpos, s));
-  PSE_TRY(gather_in(c, dF, dS, c->d_v[0], s));
+  PSE_TRY(gather_in(c, dF, dS, c->d_v[0], true, s));
   int mode = M_FULL;
   if (!E) mode = dF ? M_FSU : M_SU;
   else if (!dF && !U) mode = M_SE;
-  PSE_TRY(mobility(c, c->d_v[0], c->d_v[1], mode, parts, s));
+  if (parts & PSE_PART_REAL) PSE_TRY(real_apply(c, c->d_v[0], c->d_v[1], mode, s, true));
+  if (parts & PSE_PART_WAVE) PSE_TRY(wave_apply(c, c->d_v[0], c->d_v[1], mode, (parts & PSE_PART_REAL) != 0, s));
   PSE_TRY(scatter_out(c, c->d_v[1], dU, dE, 1.0, s));
   PSE_TRY(unstage(c, U, dU, c->ts * 3 * N, s));
   PSE_TRY(unstage(c, E, dE, c->ts * 5 * N, s));
@@ -1535,9 +1551,10 @@ pse_status pse_brownian_sample(pse_handle h, const double *pos, double dt, uint6
   PSE_TRY(scatter_out(c, c->d_v[2], dU, dE, std::sqrt(2.0 * p.kT / dt), s));
   PSE_TRY(unstage(c, UB, dU, c->ts * 3 * N, s));
   PSE_TRY(unstage(c, EB, dE, c->ts * 5 * N, s));
+  PSE_TRY(queue_krylov_stats(c, 0, s));
   PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
   c->h2d_pending = false;
-  pse_status st = read_krylov_stats(c, true, false, s);
+  pse_status st = take_krylov_stats(c, 0, true, false);
   gather_stats(c, stats);
   return st;
 }

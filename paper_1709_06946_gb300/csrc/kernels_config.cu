@@ -97,7 +97,7 @@ __device__ __forceinline__ int support_start(double x, double h, double ih, int 
 // the 4 x 4 x 4 sub-block of the tile (so that the sorted order is spatially
 // coherent inside a tile: neighbours' records then lie close together).
 __global__ void k_bin(const SysDev *__restrict__ sys, const int64_t *__restrict__ p0, int nsys, int64_t Ntot,
-                      int P, const double *pos, double *posw, int *tile_key, int *tile_cnt, int *bad) {
+                      int P, const double *pos, double *posw, int *tile_key, int *rank, int *tile_cnt, int *bad) {
   int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (u >= Ntot) return;
   const SysDev &b = sys[find_sys(p0, nsys, u)];
@@ -128,7 +128,7 @@ __global__ void k_bin(const SysDev *__restrict__ sys, const int64_t *__restrict_
             (iw[0] % b.T[0]) * SUB_SIDE / b.T[0];
   tk = tk * SUB_BLOCKS + sub;
   tile_key[u] = tk;
-  atomicAdd(&tile_cnt[tk], 1);
+  rank[u] = atomicAdd(&tile_cnt[tk], 1);
 }
 
 // tile_start[t] = fine_start[t * SUB_BLOCKS] for t = 0 .. ntiles
@@ -137,11 +137,10 @@ __global__ void k_tile_starts(int64_t ntiles, const int *fine_start, int *tile_s
   if (t <= ntiles) tile_start[t] = fine_start[t * SUB_BLOCKS];
 }
 
-__global__ void k_scatter(int64_t N, const int *key, const int *start, int *cur, int *perm, int *inv) {
+__global__ void k_scatter(int64_t N, const int *key, const int *start, const int *rank, int *perm, int *inv) {
   int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (u >= N) return;
-  int k = key[u];
-  int i = start[k] + atomicAdd(&cur[k], 1);
+  const int i = start[key[u]] + rank[u];
   perm[i] = (int)u;
   inv[u] = i;
 }
@@ -149,7 +148,7 @@ __global__ void k_scatter(int64_t N, const int *key, const int *start, int *cur,
 template <typename T>
 __global__ void k_derive(const SysDev *__restrict__ sys, const int64_t *__restrict__ p0, int nsys, int64_t Ntot,
                          int P, const int *perm, const double *posw, int4 *sp_i0, typename V4<T>::t *sp_d0,
-                         void *rs, int *cell_key, int *cell_cnt) {
+                         void *rs, int *cell_key, int *rank, int *cell_cnt) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Ntot) return;
   const SysDev &b = sys[find_sys(p0, nsys, i)];
@@ -179,19 +178,18 @@ __global__ void k_derive(const SysDev *__restrict__ sys, const int64_t *__restri
   }
   int ck = b.cell0 + (c[2] * b.nc + c[1]) * b.nc + c[0];
   cell_key[i] = ck;
-  atomicAdd(&cell_cnt[ck], 1);
+  rank[i] = atomicAdd(&cell_cnt[ck], 1);
 }
 
 // Cell list: the particles of every cell, and a copy of their records (cell
 // offsets or positions) in the same order, so that the neighbour search reads
 // contiguous records.
 template <typename T>
-__global__ void k_cell_scatter(int64_t N, int *cell_key, const int *start, int *cur, int *list,
+__global__ void k_cell_scatter(int64_t N, int *cell_key, const int *start, const int *rank, int *list,
                                const typename V4<T>::t *rs, typename V4<T>::t *rs_cell) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  int ck = cell_key[i];
-  const int k = start[ck] + atomicAdd(&cur[ck], 1);
+  const int k = start[cell_key[i]] + rank[i];
   list[k] = (int)i;
   rs_cell[k] = rs[i];
   cell_key[i] = k;  // from here on: the particle's own position in the cell list
@@ -534,48 +532,48 @@ int64_t layout_neighbours(pse_ctx *c) {
 // Builds the sorted configuration for positions d_pos (device, user order, FP64).
 pse_status setup_config(pse_ctx *c, const double *d_pos, cudaStream_t s) {
   StageTimer timer(c, PSE_STAGE_SETUP, s);
-  c->nlaunch += 6;  // bin, scatter, derive, cell scatter, neighbour count and fill (+ scans)
+  c->nlaunch += 5;  // bin, scatter, derive, cell scatter, neighbour list (+ scans)
   const Params &p = c->p;
   const int64_t N = p.N;
   const int ns = c->nsys;
   unsigned nb = (unsigned)ceil_div(N, 256);
   const int64_t nfine = c->ntiles * SUB_BLOCKS;
-  PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_fine_start, 0, sizeof(int) * (nfine + 1), s));
-  PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_fine_cur, 0, sizeof(int) * (nfine + 1), s));
-  PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_cell_start, 0, sizeof(int) * (c->ncells + 1), s));
-  PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_cell_cur, 0, sizeof(int) * (c->ncells + 1), s));
-  if (!c->capturing) PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_flag, 0, sizeof(int), s));  // a graph clears it once
-  k_bin<<<nb, 256, 0, s>>>(c->d_sys, c->d_p0, ns, N, p.P, d_pos, c->d_posw, c->d_tile_key, c->d_fine_start,
+  // status words (a graph clears them once, for both of its builds), totals and counts
+  char *clear = c->capturing ? (char *)c->d_nbr_tot : (char *)c->d_flag;
+  PSE_CUDA_TRY(c, cudaMemsetAsync(clear, 0, (char *)(c->d_cell_start + c->ncells + 1) - clear, s));
+  k_bin<<<nb, 256, 0, s>>>(c->d_sys, c->d_p0, ns, N, p.P, d_pos, c->d_posw, c->d_tile_key, c->d_rank, c->d_fine_start,
                            c->d_flag);
   PSE_TRY(exclusive_scan(c, c->d_fine_start, nfine + 1, s));
-  k_scatter<<<nb, 256, 0, s>>>(N, c->d_tile_key, c->d_fine_start, c->d_fine_cur, c->d_perm, c->d_inv);
-  k_tile_starts<<<(unsigned)ceil_div(c->ntiles + 1, 256), 256, 0, s>>>(c->ntiles, c->d_fine_start, c->d_tile_start);
+  k_scatter<<<nb, 256, 0, s>>>(N, c->d_tile_key, c->d_fine_start, c->d_rank, c->d_perm, c->d_inv);
+  if (c->n_cubic < ns) {
+    c->nlaunch += 1;
+    k_tile_starts<<<(unsigned)ceil_div(c->ntiles + 1, 256), 256, 0, s>>>(c->ntiles, c->d_fine_start, c->d_tile_start);
+  }
   if (c->prec == PSE_MIXED)
     k_derive<float><<<nb, 256, 0, s>>>(c->d_sys, c->d_p0, ns, N, p.P, c->d_perm, c->d_posw, (int4 *)c->d_sp_i0,
-                                       (float4 *)c->d_sp_d0, c->d_rs, c->d_cell_key, c->d_cell_start);
+                                       (float4 *)c->d_sp_d0, c->d_rs, c->d_cell_key, c->d_rank, c->d_cell_start);
   else
     k_derive<double><<<nb, 256, 0, s>>>(c->d_sys, c->d_p0, ns, N, p.P, c->d_perm, c->d_posw, (int4 *)c->d_sp_i0,
-                                        (double4_32a *)c->d_sp_d0, c->d_rs, c->d_cell_key, c->d_cell_start);
+                                        (double4_32a *)c->d_sp_d0, c->d_rs, c->d_cell_key, c->d_rank, c->d_cell_start);
   PSE_TRY(exclusive_scan(c, c->d_cell_start, c->ncells + 1, s));
   if (c->prec == PSE_MIXED)
-    k_cell_scatter<float><<<nb, 256, 0, s>>>(N, c->d_cell_key, c->d_cell_start, c->d_cell_cur, c->d_cell_list,
+    k_cell_scatter<float><<<nb, 256, 0, s>>>(N, c->d_cell_key, c->d_cell_start, c->d_rank, c->d_cell_list,
                                              (const float4 *)c->d_rs, (float4 *)c->d_rs_cell);
   else
-    k_cell_scatter<double><<<nb, 256, 0, s>>>(N, c->d_cell_key, c->d_cell_start, c->d_cell_cur, c->d_cell_list,
+    k_cell_scatter<double><<<nb, 256, 0, s>>>(N, c->d_cell_key, c->d_cell_start, c->d_rank, c->d_cell_list,
                                               (const double4_32a *)c->d_rs, (double4_32a *)c->d_rs_cell);
   const double rc2 = p.rcut * p.rcut;
   for (int attempt = 0; attempt < 2; ++attempt) {
-    PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_nbr_tot, 0, 2 * sizeof(unsigned long long) * ns, s));
+    if (attempt > 0) PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_nbr_tot, 0, 2 * sizeof(unsigned long long) * ns, s));
     const bool def = c->lattice != 0;
     if (c->prec == PSE_MIXED) launch_nbr<float>(c, def ? k_nbr<float, true> : k_nbr<float, false>, rc2, s);
     else launch_nbr<double>(c, def ? k_nbr<double, true> : k_nbr<double, false>, rc2, s);
     if (c->capturing) return PSE_OK;  // the graph's caller checks the flags and the totals afterwards
-    PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_pinned_int + 1, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-    PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_nbr_tot, c->d_nbr_tot, 2 * sizeof(unsigned long long) * ns,
+    PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_status, c->d_flag, 16 + 2 * sizeof(unsigned long long) * ns,
                                     cudaMemcpyDeviceToHost, s));
     PSE_CUDA_TRY(c, cudaGetLastError());
     PSE_CUDA_TRY(c, cudaStreamSynchronize(s));
-    if (c->h_pinned_int[1]) {
+    if (c->h_status[0]) {
       c->err = "non-finite particle position";
       return PSE_ERR_NONFINITE;
     }

@@ -16,20 +16,66 @@
 namespace pse {
 namespace {
 
+// Sorted rows from user-order F and S (NULL: zero); with vcell also into cell-list order as the
+// pair sum reads them (pos: a particle's place in that list).
 template <typename T>
-__global__ void k_gather_in(int64_t N, const int *perm, const T *F, const T *S, T *out) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_gather_in(int64_t N, const int *perm, const T *F, const T *S, T *out, T *vcell, const int *pos) {
+  using T4 = typename V4<T>::t;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  int u = perm[i];
-  T *o = out + 8 * (size_t)i;
-  for (int m = 0; m < 3; ++m) o[m] = F ? F[3 * (size_t)u + m] : (T)0;
-  for (int m = 0; m < 5; ++m) o[3 + m] = S ? S[5 * (size_t)u + m] : (T)0;
+  const int64_t u = perm[i];
+  T v[8];
+#pragma unroll
+  for (int m = 0; m < 3; ++m) v[m] = F ? F[3 * u + m] : (T)0;
+#pragma unroll
+  for (int m = 0; m < 5; ++m) v[3 + m] = S ? S[5 * u + m] : (T)0;
+  T4 lo, hi;
+  lo.x = v[0], lo.y = v[1], lo.z = v[2], lo.w = v[3];
+  hi.x = v[4], hi.y = v[5], hi.z = v[6], hi.w = v[7];
+  store_row((T4 *)out, i, lo, hi);
+  if (vcell) {
+    cell_row(lo, hi);
+    store_row((T4 *)vcell, pos[i], lo, hi);
+  }
+}
+
+// out = [F (user order, NULL: 0), slots 3..7 of s8 (sorted)]
+template <typename T>
+__global__ void k_gather_join(int64_t N, const int *perm, const T *F, const T *s8, T *out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 8 * N) return;
+  const int64_t i = e >> 3;
+  const int m = (int)(e & 7);
+  out[e] = m < 3 ? (F ? F[3 * (int64_t)perm[i] + m] : (T)0) : s8[e];
+}
+
+// out = [0, -(slots 3..7 of v) - (those of sub)]; rows of v through perm when it is given
+template <typename T>
+__global__ void k_rhs(int64_t N, const int *perm, const T *v, const T *sub, T *out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 8 * N) return;
+  const int64_t i = e >> 3;
+  const int m = (int)(e & 7);
+  T x = 0;
+  if (m >= 3) {
+    x = -v[8 * (perm ? (int64_t)perm[i] : i) + m];
+    if (sub) x -= sub[e];
+  }
+  out[e] = x;
+}
+
+// Status words (kernels_config.cu): non-finite positions, list overflow, non-finite inputs.
+__device__ __forceinline__ bool status_set(const int *flag) { return flag && (flag[0] | flag[1] | flag[2]); }
+
+__global__ void k_commit(int64_t n, const double *__restrict__ src, double *__restrict__ dst, const int *flag) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < n && !status_set(flag)) dst[e] = src[e];
 }
 
 template <typename T>
-__global__ void k_scatter_out(int64_t N, const int *perm, const T *in, T *U, T *E, T scale) {
+__global__ void k_scatter_out(int64_t N, const int *perm, const T *in, T *U, T *E, T scale, const int *flag) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
+  if (i >= N || status_set(flag)) return;
   int u = perm[i];
   const T *v = in + 8 * (size_t)i;
   if (U)
@@ -155,32 +201,6 @@ __global__ void k_combine(VecArgs va, T *w, const T *__restrict__ rows, int64_t 
   }
 }
 
-// dst = f * src with f = a, or f = coef[s][0] per suspension when coef is given
-template <typename T>
-__global__ void k_vscale(VecArgs va, T *dst, const T *src, T a, const double *__restrict__ coef) {
-  using V = V16<T>;
-  using VT = typename V::t;
-  const Chunk ch = chunk_of(va);
-  if (!va.active[ch.s]) return;
-  const T f = coef ? (T)coef[(size_t)ch.s * COEF_STRIDE] : a;
-  for (int64_t e = ch.beg + (int64_t)threadIdx.x * V::n; e < ch.end; e += (int64_t)blockDim.x * V::n) {
-    T x[V::n];
-    V::get(*(const VT *)(src + e), x);
-#pragma unroll
-    for (int i = 0; i < V::n; ++i) x[i] *= f;
-    *(VT *)(dst + e) = V::put(x);
-  }
-}
-
-template <typename T>
-__global__ void k_zero_slots(T *v, int64_t N, int slot0, int nslot) {
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= N * nslot) return;
-  int64_t i = e / nslot;
-  int c = (int)(e % nslot);
-  v[8 * (size_t)i + slot0 + c] = 0;
-}
-
 __device__ __forceinline__ double wrapL(double x, double L) {
   if (x >= 0.0 && x < L) return x;  // already inside: fmod would return x itself
   x = fmod(x, L);
@@ -288,12 +308,42 @@ unsigned grid_for(int64_t n, int nt = 256) { return (unsigned)ceil_div(n, nt); }
 
 int *next_queue(pse_ctx *c) { return c->d_queue + (c->queue_slot++ & 63); }
 
-pse_status gather_in(pse_ctx *c, const void *F, const void *S, void *vout, cudaStream_t s) {
+pse_status gather_in(pse_ctx *c, const void *F, const void *S, void *vout, bool cells, cudaStream_t s) {
   StageTimer timer(c, PSE_STAGE_VECTOR, s);
   c->nlaunch += 1;
   int64_t N = c->p.N;
-  DISPATCH(c, (k_gather_in<float><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const float *)F, (const float *)S, (float *)vout)),
-           (k_gather_in<double><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const double *)F, (const double *)S, (double *)vout)));
+  void *vc = cells ? c->d_vcell : nullptr;
+  DISPATCH(c, (k_gather_in<float><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const float *)F, (const float *)S, (float *)vout, (float *)vc, c->d_cell_key)),
+           (k_gather_in<double><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const double *)F, (const double *)S, (double *)vout, (double *)vc, c->d_cell_key)));
+  PSE_CUDA_TRY(c, cudaGetLastError());
+  return PSE_OK;
+}
+
+pse_status gather_join(pse_ctx *c, const void *F, const void *s8, void *vout, cudaStream_t s) {
+  StageTimer timer(c, PSE_STAGE_VECTOR, s);
+  c->nlaunch += 1;
+  int64_t N = c->p.N;
+  DISPATCH(c, (k_gather_join<float><<<grid_for(8 * N), 256, 0, s>>>(N, c->d_perm, (const float *)F, (const float *)s8, (float *)vout)),
+           (k_gather_join<double><<<grid_for(8 * N), 256, 0, s>>>(N, c->d_perm, (const double *)F, (const double *)s8, (double *)vout)));
+  PSE_CUDA_TRY(c, cudaGetLastError());
+  return PSE_OK;
+}
+
+pse_status krylov_rhs(pse_ctx *c, const void *v8, bool user, const void *sub8, void *vout, cudaStream_t s) {
+  StageTimer timer(c, PSE_STAGE_VECTOR, s);
+  c->nlaunch += 1;
+  int64_t N = c->p.N;
+  const int *perm = user ? c->d_perm : nullptr;
+  DISPATCH(c, (k_rhs<float><<<grid_for(8 * N), 256, 0, s>>>(N, perm, (const float *)v8, (const float *)sub8, (float *)vout)),
+           (k_rhs<double><<<grid_for(8 * N), 256, 0, s>>>(N, perm, (const double *)v8, (const double *)sub8, (double *)vout)));
+  PSE_CUDA_TRY(c, cudaGetLastError());
+  return PSE_OK;
+}
+
+pse_status commit_positions(pse_ctx *c, const double *src, double *dst, cudaStream_t s) {
+  StageTimer timer(c, PSE_STAGE_VECTOR, s);
+  c->nlaunch += 1;
+  k_commit<<<grid_for(3 * c->p.N), 256, 0, s>>>(3 * c->p.N, src, dst, c->d_flag);
   PSE_CUDA_TRY(c, cudaGetLastError());
   return PSE_OK;
 }
@@ -318,12 +368,13 @@ pse_status scatter12(pse_ctx *c, const void *vin, void *U, void *Om, void *E, cu
   return PSE_OK;
 }
 
-pse_status scatter_out(pse_ctx *c, const void *vin, void *U, void *E, double scale, cudaStream_t s) {
+pse_status scatter_out(pse_ctx *c, const void *vin, void *U, void *E, double scale, cudaStream_t s, bool guard) {
   StageTimer timer(c, PSE_STAGE_VECTOR, s);
   c->nlaunch += 1;
   int64_t N = c->p.N;
-  DISPATCH(c, (k_scatter_out<float><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const float *)vin, (float *)U, (float *)E, (float)scale)),
-           (k_scatter_out<double><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const double *)vin, (double *)U, (double *)E, scale)));
+  const int *flag = guard ? c->d_flag : nullptr;
+  DISPATCH(c, (k_scatter_out<float><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const float *)vin, (float *)U, (float *)E, (float)scale, flag)),
+           (k_scatter_out<double><<<grid_for(N), 256, 0, s>>>(N, c->d_perm, (const double *)vin, (double *)U, (double *)E, scale, flag)));
   PSE_CUDA_TRY(c, cudaGetLastError());
   return PSE_OK;
 }
@@ -389,28 +440,6 @@ pse_status combine_set(pse_ctx *c, void *y, const void *rows, const int *d_nrows
   c->nlaunch += 1;
   DISPATCH(c, (k_combine<float, true><<<nb, 256, 0, s>>>(va, (float *)y, (const float *)rows, n, maxrows, d_nrows, c->d_coef + off, 1.0f)),
            (k_combine<double, true><<<nb, 256, 0, s>>>(va, (double *)y, (const double *)rows, n, maxrows, d_nrows, c->d_coef + off, 1.0)));
-  PSE_CUDA_TRY(c, cudaGetLastError());
-  return PSE_OK;
-}
-
-pse_status vscale(pse_ctx *c, void *dst, const void *src, double a, int off, cudaStream_t s) {
-  StageTimer timer(c, PSE_STAGE_VECTOR, s);
-  c->nlaunch += 1;
-  const unsigned nb = (unsigned)c->nvblk;
-  VecArgs va = vec_args(c);
-  const double *cf = off >= 0 ? c->d_coef + off : nullptr;
-  DISPATCH(c, (k_vscale<float><<<nb, 256, 0, s>>>(va, (float *)dst, (const float *)src, (float)a, cf)),
-           (k_vscale<double><<<nb, 256, 0, s>>>(va, (double *)dst, (const double *)src, a, cf)));
-  PSE_CUDA_TRY(c, cudaGetLastError());
-  return PSE_OK;
-}
-
-pse_status vzero_slots(pse_ctx *c, void *v, int slot0, int nslot, cudaStream_t s) {
-  StageTimer timer(c, PSE_STAGE_VECTOR, s);
-  c->nlaunch += 1;
-  int64_t N = c->p.N;
-  DISPATCH(c, (k_zero_slots<float><<<grid_for(N * nslot), 256, 0, s>>>((float *)v, N, slot0, nslot)),
-           (k_zero_slots<double><<<grid_for(N * nslot), 256, 0, s>>>((double *)v, N, slot0, nslot)));
   PSE_CUDA_TRY(c, cudaGetLastError());
   return PSE_OK;
 }

@@ -460,18 +460,15 @@ pse_status fft(pse_ctx *c, bool forward, int comps, cudaStream_t s, int variant 
   return PSE_OK;
 }
 
+// Components spread and interpolated by a product.
+int comps_in(int mode) { return mode == M_SE || mode == M_SU ? 5 : 8; }
+int comps_out(int mode) { return mode == M_FULL ? 8 : (mode == M_SE ? 5 : 3); }
+
+// From the spread grids to the outputs: transforms, scaling, interpolation (added to vout).
 template <typename T>
-pse_status wave_apply_t(pse_ctx *c, const void *vin, void *vout, int mode, bool add, cudaStream_t s) {
+pse_status wave_finish_t(pse_ctx *c, void *vout, int mode, cudaStream_t s) {
   WaveArgs a = wave_args(c);
-  if (!add) PSE_CUDA_TRY(c, cudaMemsetAsync(vout, 0, sizeof(T) * 8 * (size_t)c->p.N, s));
-  int cin = (mode == M_SE || mode == M_SU) ? 5 : 8, cout = mode == M_FULL ? 8 : (mode == M_SE ? 5 : 3);
-  {
-    StageTimer timer(c, PSE_STAGE_SPREAD, s, mode);
-    c->nlaunch += 1;
-    spread_launch(c, a, vin, mode, s);
-  }
-  PSE_CUDA_TRY(c, cudaGetLastError());
-  PSE_TRY(fft<T>(c, true, cin, s, mode));
+  PSE_TRY(fft<T>(c, true, comps_in(mode), s, mode));
   ScaleArgs sa = scale_args(c);
   using C2 = typename Cx<T>::t;
   {
@@ -485,7 +482,7 @@ pse_status wave_apply_t(pse_ctx *c, const void *vin, void *vout, int mode, bool 
     else k_scale<T, M_FSU, NP><<<nb, 256, 0, s>>>(sa, (C2 *)c->d_cgrid);
   }
   PSE_CUDA_TRY(c, cudaGetLastError());
-  PSE_TRY(fft<T>(c, false, cout, s, mode));
+  PSE_TRY(fft<T>(c, false, comps_out(mode), s, mode));
   {
     StageTimer timer(c, PSE_STAGE_INTERP, s, mode);
     c->nlaunch += 1;
@@ -563,9 +560,22 @@ WaveArgs wave_args(const pse_ctx *c) {
   return a;
 }
 
+pse_status wave_spread(pse_ctx *c, const void *vin, int mode, cudaStream_t s) {
+  StageTimer timer(c, PSE_STAGE_SPREAD, s, mode);
+  c->nlaunch += 1;
+  spread_launch(c, wave_args(c), vin, mode, s);
+  PSE_CUDA_TRY(c, cudaGetLastError());
+  return PSE_OK;
+}
+
+pse_status wave_finish(pse_ctx *c, void *vout, int mode, cudaStream_t s) {
+  return c->prec == PSE_MIXED ? wave_finish_t<float>(c, vout, mode, s) : wave_finish_t<double>(c, vout, mode, s);
+}
+
 pse_status wave_apply(pse_ctx *c, const void *vin, void *vout, int mode, bool add, cudaStream_t s) {
-  return c->prec == PSE_MIXED ? wave_apply_t<float>(c, vin, vout, mode, add, s)
-                              : wave_apply_t<double>(c, vin, vout, mode, add, s);
+  if (!add) PSE_CUDA_TRY(c, cudaMemsetAsync(vout, 0, c->ts * 8 * (size_t)c->p.N, s));
+  PSE_TRY(wave_spread(c, vin, mode, s));
+  return wave_finish(c, vout, mode, s);
 }
 
 pse_status wave_noise(pse_ctx *c, const void *w2, uint64_t seed, uint64_t counter, void *vout, cudaStream_t s) {

@@ -166,6 +166,7 @@ struct FftGroup {
 // SMs; 2048 (250 blocks) take 17.5 us per pass over 11 rows and 1024 (500 blocks, more
 // FP64 reduction work) 21.4 us.
 constexpr int VEC_CHUNK_MAX = 16384, VEC_CHUNK_MIN = 1024, VEC_BLOCKS = 152;
+constexpr int STAT_SLOTS = 4;      // Krylov solves of one call, whose statistics are read at its end
 constexpr int COEF_STRIDE = 512;   // doubles of Krylov coefficients per suspension
 constexpr int MAX_ROWS = 128;      // Krylov vectors per dot-product / combination launch
 constexpr int CUBE_TILE = 16;      // tile side of the specialised spreading / interpolation kernels
@@ -186,6 +187,7 @@ struct KDev {
   double *coef;
   int *active, *nrows, *iter, *flag;   // flag[0]: continue the loop
   double *l_alpha, *l_beta, *l_cprev, *l_c, *l_work, *l_b0, *l_err;
+  double *stats;  // the statistics in one block: l_err, g_rel (nsys reals each), l_it, l_capped, g_it, g_capped (ints)
   const double *l_nodes;               // nodes, then weights, of the rational square root
   int *l_it, *l_capped;
   double *g_H, *g_cs, *g_sn, *g_g, *g_beta, *g_rel;
@@ -242,9 +244,11 @@ struct pse_ctx {
   double *d_posw = nullptr;     // wrapped positions, user order, N x 3
   int *d_tile_key = nullptr, *d_cell_key = nullptr;
   int *d_perm = nullptr, *d_inv = nullptr;   // sorted -> user, user -> sorted
-  int *d_tile_start = nullptr, *d_tile_cur = nullptr;   // ntiles + 1
-  int *d_fine_start = nullptr, *d_fine_cur = nullptr;   // ntiles * SUB_BLOCKS + 1 (sort by tile and sub-block)
-  int *d_cell_start = nullptr, *d_cell_cur = nullptr;   // ncells + 1
+  int *d_rank = nullptr;        // a particle's place in its bin (sort by tile, then by cell)
+  int *d_tile_start = nullptr;  // ntiles + 1 (general interpolation kernels)
+  // one block, cleared by one launch per configuration: status words, neighbour totals, bin
+  // counts of the sort by tile and sub-block (ntiles * SUB_BLOCKS + 1) and of the cells (ncells + 1)
+  int *d_fine_start = nullptr, *d_cell_start = nullptr;
   int *d_cell_list = nullptr;
   void *d_vcell = nullptr;     // the input vector of a real-space product in cell-list order (8N reals)
   void *d_rfd = nullptr;       // RFD step work space (4 x 8N reals, user order), allocated on first use
@@ -258,7 +262,8 @@ struct pse_ctx {
   int64_t nbr_cap = 0, npairs = 0, npairs_est = 0;  // last list's pairs; estimate from the densities
   std::vector<int64_t> npairs_sys;
   unsigned long long *d_nbr_tot = nullptr;  // per suspension: total pairs and maximum count
-  unsigned long long *h_nbr_tot = nullptr;  // pinned copy
+  int *h_status = nullptr;      // pinned copy of the four status words and the neighbour totals behind them
+  unsigned long long *h_nbr_tot = nullptr;  // the totals in it
   void *d_sp_i0 = nullptr;      // int4 per particle: wrapped support start
   void *d_sp_d0 = nullptr;      // real4: i0*h - x per dimension
   void *d_rs = nullptr;         // float4 (cell offset, x cell index) or double4_32a positions
@@ -266,7 +271,7 @@ struct pse_ctx {
   int64_t ntiles = 0, ncells = 0;
   int64_t tile_cap = 0, scan_cap = 0;  // allocated tile-array and scan-scratch capacities
   int *d_flag = nullptr;        // device status word
-  int *h_pinned_int = nullptr;  // host pinned scratch: 8 words, then active and row-count staging (2 x nsys)
+  int *h_pinned_int = nullptr;  // host pinned scratch
 
   // grids
   void *d_grid = nullptr;       // real grids of all suspensions (FftGroup layout)
@@ -280,8 +285,8 @@ struct pse_ctx {
   void *d_basis = nullptr;      // Krylov basis (max+1) x 8N
   double *d_dots = nullptr;     // per-block partial dot products
   double *d_coef = nullptr;     // per suspension COEF_STRIDE doubles: dots and combination coefficients
-  double *h_dots = nullptr;     // pinned, nsys x COEF_STRIDE (device-to-host)
-  double *h_wbuf = nullptr;     // pinned, nsys x COEF_STRIDE (host-to-device)
+  double *h_stats = nullptr;    // pinned copies of the Krylov statistics (KDev::stats), STAT_SLOTS of them
+  bool act_ones = false;        // every suspension is marked active (stream order)
   bool h2d_pending = false;     // a host-to-device copy from pinned staging may still be queued
 
   double *d_pos0 = nullptr, *d_posh = nullptr;  // FP64 positions, user order
@@ -289,7 +294,8 @@ struct pse_ctx {
   size_t stage_bytes[8] = {0};
   int *d_nrows = nullptr;       // per suspension: vectors in the final Krylov combination
   pse::KDev kd{};               // Krylov control state (device arrays)
-  int *h_flag = nullptr;        // pinned copy of kd.flag and kd.active
+  int *h_flag = nullptr;        // pinned copies of kd.flag and kd.active, one per iteration in flight
+  cudaEvent_t flag_ev[2] = {nullptr, nullptr};  // recorded behind them
   void *d_vin = nullptr;        // current Krylov vector, input of the products
   double *d_posout = nullptr;   // FP64 positions after a step (user order)
   bool capturing = false;       // a CUDA graph of the step is being captured
@@ -389,6 +395,9 @@ pse_status real_apply(pse_ctx *c, const void *vin, void *vout, int mode, cudaStr
 // Harmonic overlap force of the current configuration into F (user order, N x 3).
 pse_status overlap_force(pse_ctx *c, double kspring, void *F, cudaStream_t s);
 pse_status wave_apply(pse_ctx *c, const void *vin, void *vout, int mode, bool add, cudaStream_t s);
+// Its two halves: spreading, and everything behind it (added to vout).
+pse_status wave_spread(pse_ctx *c, const void *vin, int mode, cudaStream_t s);
+pse_status wave_finish(pse_ctx *c, void *vout, int mode, cudaStream_t s);
 // 11-moment product (option torque): 12-slot rows [F, L, S] -> [U, Omega, E], sorted order
 pse_status wave_apply11(pse_ctx *c, const void *vin12, void *vout12, bool add, cudaStream_t s);
 pse_status real_apply11(pse_ctx *c, const void *vin12, void *vout12, cudaStream_t s);
@@ -397,12 +406,19 @@ pse_status wave_noise(pse_ctx *c, const void *w2, uint64_t seed, uint64_t counte
 // mode flags for real/wave products
 // M_SU: S -> U (the final velocity when there is no external force)
 enum { M_FULL = 0, M_SE = 1, M_FSU = 2, M_SU = 3 };
-pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s,
-                    bool gathered = false);
+pse_status mobility(pse_ctx *c, const void *vin, void *vout, int mode, int parts, cudaStream_t s);
 
 // vector helpers
-pse_status gather_in(pse_ctx *c, const void *F, const void *S, void *vout, cudaStream_t s);
-pse_status scatter_out(pse_ctx *c, const void *vin, void *U, void *E, double scale, cudaStream_t s);
+// cells: also into d_vcell, the input of the next pair sum
+pse_status gather_in(pse_ctx *c, const void *F, const void *S, void *vout, bool cells, cudaStream_t s);
+// vout = [F (user order, may be NULL: 0), S of the sorted vector s8]
+pse_status gather_join(pse_ctx *c, const void *F, const void *s8, void *vout, cudaStream_t s);
+// vout = [0, -(S of v8) - (S of sub8)], v8 in user order when `user`, sub8 sorted or NULL
+pse_status krylov_rhs(pse_ctx *c, const void *v8, bool user, const void *sub8, void *vout, cudaStream_t s);
+// dst = src (3N positions) unless a status word is set
+pse_status commit_positions(pse_ctx *c, const double *src, double *dst, cudaStream_t s);
+// guard: write nothing if a status word is set
+pse_status scatter_out(pse_ctx *c, const void *vin, void *U, void *E, double scale, cudaStream_t s, bool guard = false);
 pse_status gather_user8(pse_ctx *c, const void *user8, void *vout, cudaStream_t s);
 pse_status scatter_user8(pse_ctx *c, const void *vin, void *user8, double scale, cudaStream_t s);
 pse_status philox_w1(pse_ctx *c, uint64_t seed, uint64_t counter, void *vout, cudaStream_t s);
@@ -412,9 +428,6 @@ pse_status philox_w1(pse_ctx *c, uint64_t seed, uint64_t counter, void *vout, cu
 pse_status combine_sub(pse_ctx *c, void *w, const void *rows, int nrows, int off, cudaStream_t s);
 pse_status combine_set(pse_ctx *c, void *y, const void *rows, const int *d_nrows, int maxrows, int off,
                        cudaStream_t s);
-// dst = a * src (a uniform) or dst = coef[s][off] * src per suspension when off >= 0.
-pse_status vscale(pse_ctx *c, void *dst, const void *src, double a, int off, cudaStream_t s);
-pse_status vzero_slots(pse_ctx *c, void *v, int slot0, int nslot, cudaStream_t s);
 pse_status midpoint(pse_ctx *c, const double *x0, const void *B_user, double fac, double *xout,
                     cudaStream_t s);
 pse_status final_update(pse_ctx *c, const double *x0, const void *B_user, const void *U_sorted,
