@@ -114,17 +114,6 @@ __device__ __forceinline__ void lookup(const double *tab, const RealArgs &a, dou
     f[k] = w0 * __ldg(r0 + k) + w1 * __ldg(r0 + 8 + k) + w2 * __ldg(r0 + 16 + k) + w3 * __ldg(r0 + 24 + k);
 }
 
-__device__ __forceinline__ float fast_rsqrt(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float fast_exp2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Function k of the fit: f_k = exp2(-cg (r - r0)^2) P_k(t), t = ta / r + tb in [-1, 1].
 __device__ __forceinline__ float poly_at(const RealPoly &p, int k, float t) {
   float v = p.c[k][POLY_DEG];
