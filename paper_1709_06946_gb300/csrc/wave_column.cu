@@ -37,6 +37,7 @@ namespace pse {
 namespace {
 
 constexpr float COL_LOG2E = 1.4426950408889634f;
+constexpr int COLQ_WARPS = 8;  // warps of a k_spread_colq CTA: one per 8 x 4 column block of a tile
 
 // Candidate ranges of the 8 source bins of a tile (see wave_cubic.cu).
 struct ColRanges {
@@ -246,10 +247,9 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), 16 / ZT == 1 ? 2 : 1)
   });
 }
 
-// Bit w set for each warp w whose column block (and z range, for ZT = 8) the P^3
-// support with start offsets (ex, ey, ez) from the tile origin overlaps, in a tile of
-// wx x wy x wz points.
-template <int NW, int ZT, int P>
+// Bit w set for each warp w whose 8 x 4 column block the P^3 support with start offsets
+// (ex, ey, ez) from the region's corner overlaps, in a region of wx x wy x wz points.
+template <int P>
 __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, int wy, int wz) {
   if (ex <= -P || ex >= wx || ey <= -P || ey >= wy || ez <= -P || ez >= wz) return 0u;
   const unsigned xm = (ex <= 7 ? 1u : 0u) | (ex + P - 1 >= 8 && wx > 8 ? 2u : 0u);
@@ -257,9 +257,7 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, 
   unsigned m = 0;
 #pragma unroll
   for (int b = 0; b < 4; ++b) m |= (b >= ylo && b <= yhi) ? xm << (2 * b) : 0u;
-  if (ZT == CUBE) return m;
-  const unsigned zm = (ez <= ZT - 1 ? 1u : 0u) | (ez + P - 1 >= ZT && wz > ZT ? 2u : 0u);
-  return ((zm & 1u) ? m : 0u) | ((zm & 2u) ? m << 8 : 0u);
+  return m;
 }
 
 // Spreading as k_spread_col, with the candidate scan shared by the CTA: in
@@ -274,6 +272,13 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, 
 // from the suspension's coefficients SysDev::qa.
 // ROW: slots per particle row of vin; COMP0: first grid component written.
 //
+// Work item: the ZT planes of one z range of a tile, with the candidates that can reach
+// them.  Half a tile on a CTA of 8 warps against the whole tile on one of 16: the halves
+// even out the last wave (216 tiles at N_g = 96) and do not wait for each other at the
+// barriers, for a quarter more candidates scanned: 8 components at N_g = 36 15.1 -> 11.8
+// us, 5 components at N_g = 96 58.0 -> 53.3, at N_g = 256 (2^20 particles) 552 -> 519 and 8
+// components 950 -> 869.  Quarters (8 rows of y) take 11.3, 59.0, 582 and 962 us.
+//
 // Bound by instruction issue.  A record carries its support start as floats and a list
 // entry is the record's offset, so that a visit needs no integer to float conversion (the
 // quarter-rate unit of the exponential) and no multiplication for the address: 5 components
@@ -283,32 +288,34 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, 
 // Tiles are 16^3 where 16 divides the grid, else as equal as possible (54 = 14 + 14 + 14 +
 // 12); columns and planes past a smaller tile's edge are idle.  Against the general
 // kernel: 5 components on 12^3 tiles at N_g = 36 65 -> 29 us (27 CTAs), the 11-moment
-// product's 8 and 3 components at N_g = 128 322 -> 120 and 199 -> 71 us.
+// product's 8 and 3 components at N_g = 128 322 -> 120 and 199 -> 71 us (103 and 61 with
+// the changes above).
 template <int C, int SLOT0, int P, int ZT, bool DEF = false, int ROW = 8, int COMP0 = 0>
-__global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ? 2 : 1)
+__global__ void __launch_bounds__(32 * COLQ_WARPS, ZT < CUBE && C <= 5 ? 4 : 2)
     k_spread_colq(WaveArgs wa, int *queue, const int4 *__restrict__ sp_i0, const float4 *__restrict__ sp_d0,
                   const float *__restrict__ vin, const int *__restrict__ fine_start, float *__restrict__ grid_all) {
-  constexpr int TS = CUBE, NW = 8 * (TS / ZT), NT = 32 * NW, RF = ColQRec<C, P>::FLOATS, CH = 2 * NT;
-  static_assert(TS % ZT == 0 && NW <= 32, "z split");
+  constexpr int PARTS = CUBE / ZT, NW = COLQ_WARPS, NT = 32 * NW, RF = ColQRec<C, P>::FLOATS, CH = 2 * NT;
+  static_assert(CUBE % ZT == 0 && CH * (RF / 4) <= 65536, "z split; record offsets of 16 bits");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float *rec = (float *)smem_raw;                                       // CH records of RF floats
   unsigned short *lists = (unsigned short *)(rec + (size_t)CH * RF);    // NW lists of up to CH slots
   __shared__ int s_cnt[2][NW];
   __shared__ ColRanges s_rng;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int wx0 = (w & 1) * 8, wy0 = ((w >> 1) & 3) * 4, wz0 = (w >> 3) * ZT;
-  const int cx = wx0 + (lane & 7), cy = wy0 + (lane >> 3);
+  const int cx = (w & 1) * 8 + (lane & 7), cy = (w >> 1) * 4 + (lane >> 3);
   const float fcx = (float)cx, fcy = (float)cy;
   const unsigned below = (1u << lane) - 1u;
-  for_each_item(queue, wa.ntiles, [&](int item) {
+  for_each_item(queue, wa.ntiles * PARTS, [&](int work) {
+    const int item = work / PARTS, z0 = (work % PARTS) * ZT;  // tile, first plane of its part
     const int si = find_sys(wa.tile0, wa.nsys, item);
     const SysDev &a = wa.sys[si];
     if (wave_skip(wa, si, a)) return;
     const int Ng = a.Ng;
     int t[3], t0[3];
     tile_of(a, item - a.tile0, t, t0);
-    const int wx = tile_width(a, t[0], 0), wy = tile_width(a, t[1], 1), wz = tile_width(a, t[2], 2);
-    if (w == 0) col_ranges(a, t, 0, wz, P, lane, fine_start, s_rng);
+    const int wx = tile_width(a, t[0], 0), wy = tile_width(a, t[1], 1), wz = min(tile_width(a, t[2], 2) - z0, ZT);
+    if (wz <= 0) return;  // a part past the edge of a smaller tile
+    if (w == 0) col_ranges(a, t, z0, wz, P, lane, fine_start, s_rng);
     if (tid < 2 * NW) (&s_cnt[0][0])[tid] = 0;
     const float nal = -(float)a.alpha * COL_LOG2E, hs = (float)a.h, pref = (float)a.pref;
     // deformed lattice: exponent coefficients (base 2) of the x-y form and of z
@@ -340,8 +347,8 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ?
         if (kk[u] >= 0) {
           ex = col_soff(i0[u].x, t0[0], Ng, P);
           ey = col_soff(i0[u].y, t0[1], Ng, P);
-          ez = col_soff(i0[u].z, t0[2], Ng, P);
-          mask = region_mask<NW, ZT, P>(ex, ey, ez, wx, wy, wz);
+          ez = col_soff(i0[u].z, t0[2], Ng, P) - z0;
+          mask = region_mask<P>(ex, ey, ez, wx, wy, wz);
         }
         const int slot = tid + u * NT;
         if (mask) {
@@ -395,7 +402,7 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ?
           q[i + 2] = u4.z;
           q[i + 3] = u4.w;
         }
-        const int pz = __float_as_int(q[4 + C + P]) - wz0;
+        const int pz = __float_as_int(q[4 + C + P]);
         // footprint point of this lane's column (exact small integers: an integer to float
         // conversion here, or a full-range exponential, costs the quarter-rate unit)
         const float jx = fcx - q[0], jy = fcy - q[1];
@@ -413,10 +420,10 @@ __global__ void __launch_bounds__(32 * 8 * (16 / ZT), (16 / ZT == 1 || C <= 5) ?
     }
     if (cx < wx && cy < wy) {
       float *grid = grid_all + a.grid0;
-      const size_t g0 = ((size_t)(t0[2] + wz0) * Ng + (t0[1] + cy)) * Ng + (t0[0] + cx);
+      const size_t g0 = ((size_t)(t0[2] + z0) * Ng + (t0[1] + cy)) * Ng + (t0[0] + cx);
 #pragma unroll
       for (int z = 0; z < ZT; ++z)
-        if (wz0 + z < wz) {
+        if (z < wz) {
 #pragma unroll
           for (int c = 0; c < C; ++c) grid[(COMP0 + c) * a.gstride + g0 + (size_t)z * Ng * Ng] = acc[z][c];
         }
@@ -555,9 +562,9 @@ void interp_col_p(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) {
 
 template <int C, int SLOT0, int P, int ZT, bool DEF = false, int ROW = 8, int COMP0 = 0>
 void launch_spread_col_z(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStream_t s) {
-  constexpr int NT = 32 * 8 * (CUBE / ZT);
   int *q = next_queue(c);
   if constexpr (!DEF && ROW == 8) if (c->opt.wave_kernel & 4) {  // every warp scans the candidates itself
+    constexpr int NT = 32 * 8 * (CUBE / ZT);
     static OccCache occ;
     auto kern = k_spread_col<C, SLOT0, P, ZT>;
     const unsigned grid = wave_grid(c, kern, 0, a.ntiles, occ, NT);
@@ -565,19 +572,20 @@ void launch_spread_col_z(pse_ctx *c, const WaveArgs &a, const void *vin, cudaStr
                              c->d_fine_start, (float *)c->d_grid);
     return;
   }
+  constexpr int NT = 32 * COLQ_WARPS;
   static std::once_flag once;
   static OccCache occ;
   auto kern = k_spread_colq<C, SLOT0, P, ZT, DEF, ROW, COMP0>;
   set_smem(kern, once);
   constexpr size_t sm = (size_t)2 * NT * ColQRec<C, P>::FLOATS * sizeof(float) +
-                        (size_t)(NT / 32) * 2 * NT * sizeof(unsigned short);
-  const unsigned grid = wave_grid(c, kern, sm, a.ntiles, occ, NT);
+                        (size_t)COLQ_WARPS * 2 * NT * sizeof(unsigned short);
+  const unsigned grid = wave_grid(c, kern, sm, a.ntiles * (CUBE / ZT), occ, NT);
   kern<<<grid, NT, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, (const float *)vin,
                             c->d_fine_start, (float *)c->d_grid);
 }
 
 // ZT: z points per thread, 8 (two z halves: 40 accumulators for 5 components,
-// two 512-thread CTAs per SM; measured 13 % faster than whole columns) by
+// four 256-thread CTAs per SM; measured 13 % faster than whole columns) by
 // default, 16 (one whole column per thread) for up to 5 components with bit 3
 // of option wave_kernel.
 template <int C, int SLOT0, int P>
