@@ -153,7 +153,7 @@ __global__ void k_combine(VecArgs va, T *w, const T *__restrict__ rows, int64_t 
   using V = V16<T>;
   using VT = typename V::t;
   __shared__ T cs[MAX_ROWS];
-  const Chunk ch = chunk_of(va);
+  const Chunk ch = chunk_of(va, blockIdx.x);
   if (!va.active[ch.s]) return;
   int nr = nrows;
   if (nrows_s) nr = min(nr, nrows_s[ch.s]);

@@ -20,11 +20,11 @@ struct VecArgs {
   int nsys, chunk;
 };
 
-__device__ __forceinline__ Chunk chunk_of(const VecArgs &va) {
+__device__ __forceinline__ Chunk chunk_of(const VecArgs &va, int b) {
   Chunk ch;
-  ch.s = find_sys(va.blk0, va.nsys, blockIdx.x);
+  ch.s = find_sys(va.blk0, va.nsys, b);
   const SysDev &q = va.sys[ch.s];
-  ch.beg = 8 * q.p0 + (int64_t)(blockIdx.x - q.blk0) * va.chunk;
+  ch.beg = 8 * q.p0 + (int64_t)(b - q.blk0) * va.chunk;
   const int64_t lim = 8 * (q.p0 + q.N);
   ch.end = ch.beg + va.chunk < lim ? ch.beg + va.chunk : lim;
   return ch;
@@ -115,7 +115,7 @@ __device__ __forceinline__ void chunk_dots(const Chunk &ch, const T *__restrict_
 // FP64 unit, one warp instruction in 16 cycles, set the time of these kernels on small
 // vectors: 31.4 -> 21.4 us per launch at N = 64000, 11 rows, 500 blocks).
 template <typename T>
-__device__ __forceinline__ void block_sums(const T acc[DOT_ROWS], int nr, double *partial, int64_t nblk, int r0,
+__device__ __forceinline__ void block_sums(const T acc[DOT_ROWS], int nr, double *partial, int64_t nblk, int b, int r0,
                                            double red[DOT_ROWS][DOT_NT / 32]) {
   static_assert(DOT_ROWS == 8 && DOT_NT == 256, "lane mapping");
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -141,7 +141,7 @@ __device__ __forceinline__ void block_sums(const T acc[DOT_ROWS], int nr, double
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     const int r = threadIdx.x >> 3;
-    if ((threadIdx.x & 7) == 0 && r < nr) partial[(r0 + r) * nblk + blockIdx.x] = sum;
+    if ((threadIdx.x & 7) == 0 && r < nr) partial[(r0 + r) * nblk + b] = sum;
   }
   __syncthreads();
 }
