@@ -315,11 +315,12 @@ def accuracy_vs_fp64(pkg, torch, dev, args, pos_np, L, h64):
 # records.  The wave-space kernels are left out (their grid bytes stay partly in L2 between launches,
 # so they do not scale with N_g^3).  Reported only for that workload.
 NCU_TRAFFIC_WORKLOAD = (1048576, 0.3, 1e-3, 0.5, 256, 6)
-NCU_TRAFFIC = {'k_real<float,M_FULL>': 1.926e9, 'k_real<float,M_SE>': 1.926e9, 'k_real<float,M_SU>': 1.892e9}
+NCU_TRAFFIC = {'k_real<float,M_FULL>': 1.764e9, 'k_real<float,M_SE>': 1.739e9}
 
 
 def real_flops_per_pair():
-    # FP32 operations of the pair kernel per neighbour, counted from its formulas (FMA = 2):
+    # FP32 operations per neighbour, counted from the formulas (FMA = 2) with the functions interpolated
+    # from their table (the polynomial form spends more on them, the Cartesian rows less on the rest):
     # separation and 1/r 10; table interpolation 2 + 3 per function (7, 3 or 4 functions);
     # S r^ 26; r^.S r^ 5; r^.F 5; U terms 22 (13 without F); E terms 87 (78 without F, two
     # Y-basis products of 24 each).  Full 8->8 product (Lanczos), S->E (GMRES), [F;S]->U and

@@ -17,7 +17,7 @@
 //
 // Bound by launch and reduction latency below about 10^5 particles and by HBM above.
 // Per GMRES iteration, all vector and control kernels, against eleven separate launches
-// on 16384-element blocks: N = 3000 63 -> 27 us, N = 64000 (11 rows) 120 -> 56 us,
+// on 16384-element blocks: N = 3000 63 -> 25 us, N = 64000 (11 rows) 120 -> 56 us,
 // N = 2^20 (4 rows) 205 -> 156 us.
 //
 // The dot products, scale factors and combination coefficients live in the

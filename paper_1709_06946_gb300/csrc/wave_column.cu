@@ -287,7 +287,7 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, 
 //
 // Tiles are 16^3 where 16 divides the grid, else as equal as possible (54 = 14 + 14 + 14 +
 // 12); columns and planes past a smaller tile's edge are idle.  Against the general
-// kernel: 5 components on 12^3 tiles at N_g = 36 65 -> 29 us (27 CTAs), the 11-moment
+// kernel: 5 components on 12^3 tiles at N_g = 36 65 -> 29 us (22 with the changes above), the 11-moment
 // product's 8 and 3 components at N_g = 128 322 -> 120 and 199 -> 71 us (103 and 61 with
 // the changes above).
 template <int C, int SLOT0, int P, int ZT, bool DEF = false, int ROW = 8, int COMP0 = 0>
