@@ -279,7 +279,8 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, 
 // us, 5 components at N_g = 96 58.0 -> 53.3, at N_g = 256 (2^20 particles) 552 -> 519 and 8
 // components 950 -> 869.  Quarters (8 rows of y) take 11.3, 59.0, 582 and 962 us.
 //
-// Bound by instruction issue.  A record carries its support start as floats and a list
+// Bound by instruction issue (62 % of the slots at N = 524288) and the barriers between
+// scan and update.  A record carries its support start as floats and a list
 // entry is the record's offset, so that a visit needs no integer to float conversion (the
 // quarter-rate unit of the exponential) and no multiplication for the address: 5 components
 // at P = 6, 2^20 particles 668 -> 549 us, 64,000 70 -> 58, 30,000 36 -> 30; P = 8 on a
