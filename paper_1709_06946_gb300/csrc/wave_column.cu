@@ -283,8 +283,8 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, 
 // scan and update.  A record carries its support start as floats and a list
 // entry is the record's offset, so that a visit needs no integer to float conversion (the
 // quarter-rate unit of the exponential) and no multiplication for the address: 5 components
-// at P = 6, 2^20 particles 668 -> 549 us, 64,000 70 -> 58, 30,000 36 -> 30; P = 8 on a
-// sheared box, 150,000 particles 155 -> 139.
+// at P = 6, 2^20 particles 668 -> 549 us, 64,000 70 -> 58, 30,000 36 -> 30; P = 8,
+// 150,000 particles 155 -> 139.
 //
 // Tiles are 16^3 where 16 divides the grid, else as equal as possible (54 = 14 + 14 + 14 +
 // 12); columns and planes past a smaller tile's edge are idle.  Against the general
