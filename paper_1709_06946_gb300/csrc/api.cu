@@ -142,9 +142,11 @@ pse_status set_all_active(pse_ctx *c, cudaStream_t s) {
 // iteration, and queues the next iteration's first part (all of it, when there is no
 // second part) before it waits for them, so the device does not idle while the host
 // wakes up and launches: 42 us per iteration for a sample of 50000 particles, 50 for a
-// step of 30000.  While the step is being captured it becomes a conditional while node
-// whose body graph is captured from a second stream, so the whole loop runs on the
-// device.
+// step of 30000.  With stage timing on it queues nothing ahead: what is queued behind the
+// last iteration runs on no suspension and would count as a call of its stages (8 pair
+// sums for 7 iterations, each made out an eighth shorter than it is).  While the step is
+// being captured it becomes a conditional while node whose body graph is captured from a
+// second stream, so the whole loop runs on the device.
 template <typename First, typename Second, typename Step>
 pse_status krylov_loop(pse_ctx *c, int cap, bool has_second, cudaStream_t s, First &&first, Second &&second,
                        Step &&step) {
@@ -158,18 +160,20 @@ pse_status krylov_loop(pse_ctx *c, int cap, bool has_second, cudaStream_t s, Fir
       PSE_CUDA_TRY(c, cudaEventRecord(c->flag_ev[j & 1], s));
       return PSE_OK;
     };
+    const bool ahead = !c->prof_on;
     PSE_TRY(first(s));
     PSE_TRY(rest(0));
     for (int j = 0; j < cap; ++j) {
       const bool more = j + 1 < cap;
-      if (more) PSE_TRY(first(s));
-      if (more && !has_second) PSE_TRY(rest(j + 1));
+      if (more && ahead) PSE_TRY(first(s));
+      if (more && ahead && !has_second) PSE_TRY(rest(j + 1));
       PSE_CUDA_TRY(c, cudaEventSynchronize(c->flag_ev[j & 1]));
       c->h2d_pending = false;
       const int *f = c->h_flag + (j & 1) * nf;
       std::copy(f + 1, f + nf, c->h_active.begin());
       if (!f[0]) break;
-      if (more && has_second) PSE_TRY(rest(j + 1));
+      if (more && !ahead) PSE_TRY(first(s));
+      if (more && (has_second || !ahead)) PSE_TRY(rest(j + 1));
     }
     return PSE_OK;
   }
