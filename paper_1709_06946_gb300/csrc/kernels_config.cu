@@ -189,7 +189,7 @@ __global__ void k_derive(const SysDev *__restrict__ sys, const int64_t *__restri
     c[d] = q.n;
     xc[d] = x[d] - q.f * b.cs;
   }
-  sp_i0[i] = make_int4(iw[0], iw[1], iw[2], 0);
+  sp_i0[i] = make_int4(iw[0], iw[1], iw[2], c[0] | (c[1] << 10) | (c[2] << 20));  // w: the cell, at most 1023 a side
   typename V4<T>::t dd;
   dd.x = d0[0];
   dd.y = d0[1];
@@ -238,7 +238,8 @@ __global__ void k_cell_scatter(int64_t N, int *cell_key, const int *start, const
 // wavefronts) and left small systems with a few warps of a long serial loop; the FP64
 // form also divided by L for every candidate.  Measured, before and after: N = 3000 155
 // -> 23 us, 64 suspensions of 160000 284 -> 196, sheared cell of 150000 465 -> 294, 2^20
-// (r_cut 7.07, 105 neighbours) 1180 -> 1037, FP64 form at 11000 1102 -> 125.
+// (r_cut 7.07, 105 neighbours) 1180 -> 1037, FP64 form at 11000 1102 -> 125.  Dilute
+// systems take k_nbr_sparse (use_sparse).
 // DEF: deformed lattice (Sec. 2.3.3): records and cells hold lattice coordinates z,
 // and each candidate's separation is mapped to x_i - x_j = A (z_i - z_j) before the
 // test, so the stored separations are Cartesian as for the cube.
@@ -268,6 +269,40 @@ __device__ __forceinline__ void add_totals(unsigned long long *tot, int si, int 
   }
 }
 
+// x_i - x_j for a particle's coordinates c and a candidate's record q; sx, sy, sz: cells (FP32) or
+// box lengths (FP64) to the nearest image.
+template <typename T, bool DEF, bool WIDE>
+__device__ __forceinline__ typename V4<T>::t nbr_sep(const T c[3], const typename V4<T>::t &q, T sx, T sy, T sz, T cs,
+                                                     T L, const T *A) {
+  typename V4<T>::t rec;
+  if (sizeof(T) == 4) {
+    rec.x = fma(sx, cs, c[0] - q.x);
+    rec.y = fma(sy, cs, c[1] - q.y);
+    rec.z = fma(sz, cs, c[2] - q.z);
+  } else {
+    rec.x = c[0] - q.x;
+    rec.y = c[1] - q.y;
+    rec.z = c[2] - q.z;
+    if (WIDE) {  // the nearest image is s box lengths away (pairs beyond it are further than r_cut)
+      rec.x -= L * sx;
+      rec.y -= L * sy;
+      rec.z -= L * sz;
+    }
+  }
+  if (!WIDE) {
+    rec.x -= L * rint(rec.x / L);
+    rec.y -= L * rint(rec.y / L);
+    rec.z -= L * rint(rec.z / L);
+  }
+  if constexpr (DEF) {  // x_i - x_j = A (z_i - z_j)
+    const T zx = rec.x, zy = rec.y, zz = rec.z;
+    rec.x = A[0] * zx + A[1] * zy + A[2] * zz;
+    rec.y = A[3] * zx + A[4] * zy + A[5] * zz;
+    rec.z = A[6] * zx + A[7] * zy + A[8] * zz;
+  }
+  return rec;
+}
+
 // The runs of one pass (lane r: start, length and y / z offsets of run r) walked for up to
 // NP particles of the cell.
 template <typename T, bool DEF, bool WIDE, int NP>
@@ -293,34 +328,8 @@ struct NbrWalk {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       if (p < np) {
-        T4 rec;
-        bool hit;
-        if (sizeof(T) == 4) {
-          rec.x = fma(sx, cs, ctr[p][0] - q.x);
-          rec.y = fma(sy, cs, ctr[p][1] - q.y);
-          rec.z = fma(sz, cs, ctr[p][2] - q.z);
-        } else {
-          rec.x = ctr[p][0] - q.x;
-          rec.y = ctr[p][1] - q.y;
-          rec.z = ctr[p][2] - q.z;
-          if (WIDE) {  // the nearest image is s box lengths away (pairs beyond it are further than r_cut)
-            rec.x -= L * sx;
-            rec.y -= L * sy;
-            rec.z -= L * sz;
-          }
-        }
-        if (!WIDE) {
-          rec.x -= L * rint(rec.x / L);
-          rec.y -= L * rint(rec.y / L);
-          rec.z -= L * rint(rec.z / L);
-        }
-        if constexpr (DEF) {  // x_i - x_j = A (z_i - z_j)
-          const T zx = rec.x, zy = rec.y, zz = rec.z;
-          rec.x = A[0] * zx + A[1] * zy + A[2] * zz;
-          rec.y = A[3] * zx + A[4] * zy + A[5] * zz;
-          rec.z = A[6] * zx + A[7] * zy + A[8] * zz;
-        }
-        hit = rec.x * rec.x + rec.y * rec.y + rec.z * rec.z < rc2 && live && k != kb + p;
+        T4 rec = nbr_sep<T, DEF, WIDE>(ctr[p], q, sx, sy, sz, cs, L, A);
+        const bool hit = rec.x * rec.x + rec.y * rec.y + rec.z * rec.z < rc2 && live && k != kb + p;
         const unsigned hits = __ballot_sync(0xffffffffu, hit);
         const int to = at[p] + __popc(hits & below);
         if (hit && to < lim[p]) {  // separation x_i - x_j and the neighbour's cell-list position
@@ -483,6 +492,79 @@ __global__ void __launch_bounds__(NBR_NT, sizeof(T) == 4 ? 4 : 1)
   if (si >= 0) add_totals(tot, si, lane, sum, big);
 }
 
+// The same list, one thread per particle, for systems of mostly empty cells (use_sparse):
+// a thread streams through the cell-ordered records of its 25 runs, NB of them loaded before
+// the first is tested.  Bound by the latency of that walk; 10^6 particles at a volume fraction of
+// 0.01 take 165 us, 983 with a warp per cell.
+template <typename T, bool DEF>
+__global__ void __launch_bounds__(128)
+    k_nbr_sparse(const SysDev *__restrict__ sys, const int64_t *__restrict__ p0, int nsys, int64_t Ntot, float rc2f,
+                 double rc2, const typename V4<T>::t *__restrict__ rs_cell, const int4 *__restrict__ sp_i0,
+                 const int *__restrict__ cell_start, const int *__restrict__ cell_pos, int *cnt, typename V4<T>::t *geo,
+                 unsigned long long *tot, int *ovf) {
+  using T4 = typename V4<T>::t;
+  constexpr int NB = 4;  // candidate records loaded before the first is tested
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= Ntot) return;
+  const int si = find_sys(p0, nsys, i), self = cell_pos[i], packed = sp_i0[i].w;
+  const SysDev &a = sys[si];
+  const int nc = a.nc, slots = a.slots, cell0 = a.cell0;
+  const T cs = sizeof(T) == 4 ? (T)a.csf : (T)a.cs, L = sizeof(T) == 4 ? (T)a.Lf : (T)a.L;
+  const T r2max = sizeof(T) == 4 ? (T)rc2f : (T)rc2;
+  T A[DEF ? 9 : 1];
+  if constexpr (DEF) {
+#pragma unroll
+    for (int m = 0; m < 9; ++m) A[m] = sizeof(T) == 4 ? (T)a.Af[m] : (T)a.A[m];
+  }
+  const int cx = packed & 1023, cy = (packed >> 10) & 1023, cz = packed >> 20;
+  const T4 own = rs_cell[self];
+  const T ctr[3] = {own.x, own.y, own.z};
+  T4 *row_geo = geo + a.nbr0 + (i - a.p0) * slots;
+  int n = 0;
+  for (int dz = -2; dz <= 2; ++dz)
+    for (int dy = -2; dy <= 2; ++dy) {
+      const int rz = cz + dz, ry = cy + dy;
+      const int wz = rz < 0 ? -1 : (rz >= nc ? 1 : 0), wy = ry < 0 ? -1 : (ry >= nc ? 1 : 0);
+      const int row = cell0 + ((rz - wz * nc) * nc + (ry - wy * nc)) * nc;
+      const T sy = sizeof(T) == 4 ? (T)-dy : (T)wy, sz = sizeof(T) == 4 ? (T)-dz : (T)wz;
+      // cells [cx - 2, cx + 2], in two ranges where they wrap
+      for (int wx = cx < 2 ? -1 : 0; wx <= (cx + 2 >= nc ? 1 : 0); ++wx) {
+        const int kb = cell_start[row + max(cx - 2 - wx * nc, 0)];
+        const int ke = cell_start[row + min(cx + 2 - wx * nc, nc - 1) + 1];
+        const T sx = sizeof(T) == 4 ? (T)(cx - wx * nc) : (T)wx;
+        for (int k = kb; k < ke; k += NB) {
+          T4 q[NB];
+#pragma unroll
+          for (int u = 0; u < NB; ++u)
+            if (k + u < ke) q[u] = rs_cell[k + u];
+#pragma unroll
+          for (int u = 0; u < NB; ++u) {
+            if (k + u >= ke) break;
+            T4 rec = nbr_sep<T, DEF, true>(ctr, q[u], sizeof(T) == 4 ? sx - (T)q[u].w : sx, sy, sz, cs, L, A);
+            if (rec.x * rec.x + rec.y * rec.y + rec.z * rec.z < r2max && k + u != self) {
+              if (n < slots) {
+                rec.w = index_as_real<T>(k + u);
+                row_geo[n] = rec;
+              }
+              ++n;
+            }
+          }
+        }
+      }
+    }
+  cnt[i] = n;
+  if (n > slots) atomicOr(ovf, 1);
+  // one atomic addition per warp when its particles share a suspension
+  const unsigned act = __activemask();
+  const int leader = __ffs(act) - 1;
+  if (__all_sync(act, si == __shfl_sync(act, si, leader))) {
+    const unsigned sum = __reduce_add_sync(act, (unsigned)n), big = __reduce_max_sync(act, (unsigned)n);
+    if ((int)(threadIdx.x & 31) == leader) add_totals(tot, si, 0, sum, (int)big);
+  } else {
+    add_totals(tot, si, 0, (unsigned)n, n);
+  }
+}
+
 void *alloc_dev(pse_ctx *c, size_t bytes) {
   void *p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
@@ -491,10 +573,33 @@ void *alloc_dev(pse_ctx *c, size_t bytes) {
   return p;
 }
 
+// One thread per particle where most cells hold one particle or none: a warp per cell then
+// has few candidates for its lanes and few particles to test them against, and walks past
+// the empty cells one after the other.  A thread's serial walk over 25 runs takes 20 us and more,
+// so there have to be many cells for it (600 per SM).  Measured, us, warp / thread:
+//   FP32  N = 10^6: 0.1 particles per cell 983 / 165, 0.86 708 / 348, 1.5 756 / 535, 2.2 860 / 734
+//         300000: 0.02 850 / 53, 0.87 230 / 133, 1.5 243 / 204, 2.1 265 / 263;  200000: 1.5 167 / 163, 1.8 174 / 205
+//         60000: 0.22 61 / 31, 0.87 55 / 51, 1.3 56 / 65;  30000: 0.11 44 / 26, 0.44 33 / 38;  10000: 0.11 21 / 23
+//   FP64  300000: 0.11 477 / 489, 0.21 435 / 686;  100000: 0.02 499 / 103;  30000: 0.02 164 / 42, 0.11 74 / 81
+bool use_sparse(const pse_ctx *c) {
+  for (const Params &p : c->ps)
+    if (p.nc < 5) return false;
+  if (c->ncells < 600 * (int64_t)c->nsm) return false;
+  return c->prec == PSE_MIXED ? 2 * c->ncells >= c->p.N + 65536 : c->ncells >= 16 * c->p.N;
+}
+
 // A warp per cell; beyond 16 blocks per SM each walks several cells, so the totals take
 // one atomic addition per warp and not per cell.
-template <typename T, typename K>
-void launch_nbr(pse_ctx *c, K kern, double rc2, cudaStream_t s) {
+template <typename T, bool DEF>
+void launch_nbr(pse_ctx *c, double rc2, cudaStream_t s) {
+  using T4 = typename V4<T>::t;
+  if (use_sparse(c)) {
+    k_nbr_sparse<T, DEF><<<(unsigned)ceil_div(c->p.N, 128), 128, 0, s>>>(
+        c->d_sys, c->d_p0, c->nsys, c->p.N, (float)rc2, rc2, (const T4 *)c->d_rs_cell, (const int4 *)c->d_sp_i0,
+        c->d_cell_start, c->d_cell_key, c->d_nbr_start, (T4 *)c->d_nbr_geo, c->d_nbr_tot, c->d_flag + 1);
+    return;
+  }
+  auto kern = k_nbr<T, DEF>;
   const int64_t nb = std::min<int64_t>(ceil_div(c->ncells, NBR_NT / 32), (int64_t)c->nsm * 16);
   kern<<<(unsigned)nb, NBR_NT, 0, s>>>(c->d_sys, c->nsys, c->ncells, (float)rc2, rc2, c->d_rs_cell, c->d_cell_start,
                                        c->d_cell_list, c->d_nbr_start, (typename V4<T>::t *)c->d_nbr_geo,
@@ -591,8 +696,8 @@ pse_status setup_config(pse_ctx *c, const double *d_pos, cudaStream_t s) {
   for (int attempt = 0; attempt < 2; ++attempt) {
     if (attempt > 0) PSE_CUDA_TRY(c, cudaMemsetAsync(c->d_nbr_tot, 0, 2 * sizeof(unsigned long long) * ns, s));
     const bool def = c->lattice != 0;
-    if (c->prec == PSE_MIXED) launch_nbr<float>(c, def ? k_nbr<float, true> : k_nbr<float, false>, rc2, s);
-    else launch_nbr<double>(c, def ? k_nbr<double, true> : k_nbr<double, false>, rc2, s);
+    if (c->prec == PSE_MIXED) def ? launch_nbr<float, true>(c, rc2, s) : launch_nbr<float, false>(c, rc2, s);
+    else def ? launch_nbr<double, true>(c, rc2, s) : launch_nbr<double, false>(c, rc2, s);
     if (c->capturing) return PSE_OK;  // the graph's caller checks the flags and the totals afterwards
     PSE_CUDA_TRY(c, cudaMemcpyAsync(c->h_status, c->d_flag, 16 + 2 * sizeof(unsigned long long) * ns,
                                     cudaMemcpyDeviceToHost, s));
