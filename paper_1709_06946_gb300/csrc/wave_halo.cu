@@ -14,8 +14,8 @@
 // Against the general kernel on 12^3 tiles at N_g = 36: 5 components 55 -> 7.4 us, 8
 // components 39 -> 8.7; the 11-moment product's at N_g = 128 187 -> 105 and 133 -> 60 us.
 // Two CTAs share an SM (about 83 KB each for 5 components, P = 6), so one CTA's
-// staging overlaps the other's read-out; with enough tiles an item is a whole tile whose
-// planes pass through a ring (halo_layers).
+// staging overlaps the other's read-out; where staging is most of the work an item is a whole
+// tile whose planes pass through a ring (halo_may_ring).
 //
 // Bound by L1: two thirds of the shared-memory and copy wavefronts of the one-layer form
 // are staging (8 per 32 four-byte copies; 3969 points for 64 particles), the rest the
@@ -27,7 +27,7 @@
 namespace pse {
 namespace {
 
-// One layer per work item: 512 threads, two CTAs per SM.  Several layers per item: 1024 threads
+// One layer per work item: 512 threads, two CTAs per SM.  A whole tile per item: 1024 threads
 // and a ring of planes, one CTA per SM.
 constexpr int HALO_THREADS = 512, RING_THREADS = 1024;
 
@@ -63,13 +63,12 @@ template <int P, bool RING = false> struct Halo {
 // COMP0: first grid component read (grid components COMP0 .. COMP0 + C - 1 go
 // to output slots SLOT0 .. SLOT0 + C - 1).  ROW: slots per particle row of vout.
 //
-// RING: an item is `nl` consecutive layers of a tile.  The planes stay in a ring of
-// slots, so a layer stages only the planes that the one below it did not have (21
+// RING: an item is a tile.  The planes stay in a ring of slots, so a layer stages only the planes that the one below it did not have (21
 // planes for the four layers of a 16^3 tile at P = 6, not 36), and they are copied while
 // the layer below is read out.
 template <int C, int SLOT0, int P, bool DEF, int COMP0, int ROW, bool RING>
 __global__ void __launch_bounds__(RING ? RING_THREADS : HALO_THREADS, RING ? 1 : 2)
-    k_interp_halo(WaveArgs wa, int *queue, int nl, const int4 *__restrict__ sp_i0, const float4 *__restrict__ sp_d0,
+    k_interp_halo(WaveArgs wa, int *queue, const int4 *__restrict__ sp_i0, const float4 *__restrict__ sp_d0,
                   const int *__restrict__ fine_start, const float *__restrict__ grid_all, float *__restrict__ vout) {
   using H = Halo<P, RING>;
   constexpr int R = H::R, NZ = H::NZ, RX = H::RX, ZS = H::ZS, LP = H::LP, NT = RING ? RING_THREADS : HALO_THREADS;
@@ -77,10 +76,9 @@ __global__ void __launch_bounds__(RING ? RING_THREADS : HALO_THREADS, RING ? 1 :
   TileL<float, C> tl;
   tl.init(smem_raw, H::NPT);
   const int lane = threadIdx.x & 31, group = lane / LP, sub = lane % LP, warp = threadIdx.x >> 5;
-  const int per_tile = RING ? (SUB_SIDE + nl - 1) / nl : SUB_SIDE;
+  constexpr int per_tile = RING ? 1 : SUB_SIDE;
   for_each_item(queue, wa.ntiles * per_tile, [&](int item) {
-    const int tile = item / per_tile, kz0 = (item % per_tile) * (RING ? nl : 1);
-    const int kz1 = RING ? min(kz0 + nl, SUB_SIDE) : kz0 + 1;
+    const int tile = item / per_tile, kz0 = item % per_tile, kz1 = RING ? SUB_SIDE : kz0 + 1;
     const int si = find_sys(wa.tile0, wa.nsys, tile);
     const SysDev &a = wa.sys[si];
     if (wave_skip(wa, si, a)) return;
@@ -95,14 +93,19 @@ __global__ void __launch_bounds__(RING ? RING_THREADS : HALO_THREADS, RING ? 1 :
     auto first = [&](int kz) { return min((kz * a.T[2] + SUB_SIDE - 1) / SUB_SIDE, wz); };
     const int rx = tile_width(a, t[0], 0) + P - 1, ry = tile_width(a, t[1], 1) + P - 1;
     const float *grid = grid_all + a.grid0 + COMP0 * a.gstride;
+    const int64_t gs = a.gstride;  // in a register: the copies keep the compiler from holding values read through `a`
     const bool whole = rx == R && ry == R;
     // planes [za, zb) (from the tile's origin, periodic) into the tile layout; plane z lies in
-    // slot z mod NZ: asynchronous 4-byte copies (no register round trip), or for 5 components
-    // and one layer per item loads and vector stores, U points per thread in flight
+    // slot z mod NZ: asynchronous 4-byte copies (no register round trip), or for 5 components,
+    // small supports and one layer per item loads and vector stores, U points per thread in
+    // flight.  Unrolled: the copies' addresses take longer than the copies (8 components, P = 8,
+    // 4096 tiles: 1123 us as a loop with gstride read per copy, 1023 so, 1057 unrolled 4; one
+    // layer of 5 components, P = 6: 422 -> 384; the ring of 5 at P = 10 3457 unrolled 2, 3070 by 4)
     auto stage = [&](int za, int zb) {
-      constexpr bool REGS = C == 5 && !RING;
-      constexpr int U = REGS ? 2 : 1;
+      constexpr bool REGS = C == 5 && P <= 6 && !RING;
+      constexpr int U = REGS ? 2 : 1, UNROLL = REGS || (C == 5 && RING) ? 4 : 2;
       const int n = (zb - za) * R * R;
+#pragma unroll UNROLL
       for (int q0 = threadIdx.x; q0 < n; q0 += U * NT) {
         float v[U][C];
         int d[U];
@@ -119,8 +122,8 @@ __global__ void __launch_bounds__(RING ? RING_THREADS : HALO_THREADS, RING ? 1 :
           if (in) {
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-              if (REGS) v[u][c] = __ldg(g + c * a.gstride);
-              else cp_async4(tl.comp(d[u], c), g + c * a.gstride);
+              if (REGS) v[u][c] = __ldg(g + c * gs);
+              else cp_async4(tl.comp(d[u], c), g + c * gs);
             }
           }
         }
@@ -228,7 +231,7 @@ constexpr size_t halo_bytes() {
 }
 
 template <int C, int SLOT0, int P, bool DEF, int COMP0, int ROW, bool RING>
-void launch_interp_halo_k(pse_ctx *c, const WaveArgs &a, void *vout, int nl, cudaStream_t s) {
+void launch_interp_halo_k(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) {
   constexpr int NT = RING ? RING_THREADS : HALO_THREADS;
   static_assert(halo_bytes<C, P, RING>() <= 223 * 1024, "staged planes");
   static std::once_flag once;
@@ -236,21 +239,22 @@ void launch_interp_halo_k(pse_ctx *c, const WaveArgs &a, void *vout, int nl, cud
   const size_t sm = TileL<float, C>::bytes((size_t)Halo<P, RING>::NPT);
   auto kern = k_interp_halo<C, SLOT0, P, DEF, COMP0, ROW, RING>;
   set_smem(kern, once);
-  const unsigned grid = wave_grid(c, kern, sm, a.ntiles * (int)ceil_div(SUB_SIDE, nl), occ, NT);
+  const unsigned grid = wave_grid(c, kern, sm, a.ntiles * (RING ? 1 : SUB_SIDE), occ, NT);
   int *q = next_queue(c);
-  kern<<<grid, NT, sm, s>>>(a, q, nl, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, c->d_fine_start,
+  kern<<<grid, NT, sm, s>>>(a, q, (const int4 *)c->d_sp_i0, (const float4 *)c->d_sp_d0, c->d_fine_start,
                             (const float *)c->d_grid, (float *)vout);
 }
 
-// Layers per item: the ring of a whole tile where there are enough tiles per SM.  Measured
-// (us, one layer / ring; 2^20 = 4096 tiles, P = 6 unless said): 8 components 126 / 105 at
-// 512 tiles, 1002 / 722 at 4096; 5 components 68 / 79 at 512, 115 / 109 at 729, 198 / 141 at
-// 729 and P = 8, 549 / 540 at 4096; 3 components 420 / 467 at 4096 (never).  A layer of a
-// ring holds about 64 particles for 128 places, so the ring gains where staging is most
-// of the work (8 components; large supports).  Two layers per item lay between.
-template <int C>
-inline int halo_layers(const pse_ctx *c, const WaveArgs &a) {
-  return a.ntiles >= (C == 8 ? 2 : 4) * c->nsm ? SUB_SIDE : 1;
+// Whether an item is a whole tile (ring) or a layer.  A layer of a ring holds about 64
+// particles for 128 places, so the ring gains where staging is most of the work: 8
+// components, and 5 with large supports, from two tiles per SM on.  Measured, us, one layer
+// / ring: 8 components, P = 6 69 / 60 at 343 tiles, 119 / 99 at 512, 931 / 673 at 4096
+// (2^20 particles); 5 components, P = 8 98 / 86 at 512 and 1234 / 950 at 5832, P = 10 139 /
+// 133 and 1847 / 1527; but P = 6 64 / 78 at 512, 384 / 446 at 4096 with 300000 particles,
+// 499 / 528 with 2^20, and P = 5 538 / 595 at 5832; 3 components 420 / 467 at 4096.
+template <int C, int P>
+constexpr bool halo_may_ring() {
+  return (C == 8 || (C == 5 && P >= 8)) && halo_bytes<C, P, true>() <= 223 * 1024;
 }
 
 template <int C, int SLOT0, int P, bool DEF, int COMP0, int ROW>
@@ -261,11 +265,9 @@ void launch_interp_halo(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t 
     launch_interp_halo<3, SLOT0 + 5, P, DEF, COMP0 + 5, ROW>(c, a, vout, s);
     c->nlaunch += 1;
   } else {
-    if constexpr (C != 3 && halo_bytes<C, P, true>() <= 223 * 1024) {
-      const int nl = halo_layers<C>(c, a);
-      if (nl > 1) return launch_interp_halo_k<C, SLOT0, P, DEF, COMP0, ROW, true>(c, a, vout, nl, s);
-    }
-    launch_interp_halo_k<C, SLOT0, P, DEF, COMP0, ROW, false>(c, a, vout, 1, s);
+    if constexpr (halo_may_ring<C, P>())
+      if (a.ntiles >= 2 * c->nsm) return launch_interp_halo_k<C, SLOT0, P, DEF, COMP0, ROW, true>(c, a, vout, s);
+    launch_interp_halo_k<C, SLOT0, P, DEF, COMP0, ROW, false>(c, a, vout, s);
   }
 }
 
