@@ -174,11 +174,14 @@ __device__ __forceinline__ void pair_terms(const T rh[3], const T row[8], const 
 // FP64 form at 11000 particles 630 -> 445 us.  Below 10^5 particles the few thousand warps
 // wait on their records (47 us at 64000, 68 before).
 //
-// FP32: 48 registers so that five 256-thread CTAs fit an SM (four: S -> E 487 us; six:
-// full 751 us, spilled).  A static split over warps instead of the work counter: full 737
-// us.  With LK_SMEM one 1024-thread CTA per SM first copies the table into shared memory.
+// FP32, polynomials: 48 registers so that five 256-thread CTAs fit an SM (four: S -> E 487
+// us; six: full 751 us, spilled).  With the table 64 registers and four, as its lookups of the
+// full product do not fit 48: per product 831 -> 803 us at 10^6 particles, 149 -> 140 at 10^5 and
+// xi = 0.3, 27 -> 21 at 3000; S -> E the same.  A static split over warps instead of the work
+// counter: full 737 us.  With LK_SMEM one 1024-thread CTA per SM first copies the table into
+// shared memory.
 template <typename T, int MODE, int G, int LK = LK_TABLE, int NT = LK == LK_SMEM ? 1024 : 256>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (LK == LK_SMEM ? 1 : 5) : 1)
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (LK == LK_SMEM ? 1 : (LK == LK_TABLE ? 4 : 5)) : 1)
     k_real(RealArgs a, RealPoly poly, const SysDev *__restrict__ sys, const int64_t *__restrict__ p0,
            const int *__restrict__ active, int *queue, int nitems, const int *__restrict__ nstart,
            const typename V4<T>::t *__restrict__ geo, const T *__restrict__ vin, const T *__restrict__ vcell,
