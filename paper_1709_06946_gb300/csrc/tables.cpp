@@ -506,11 +506,12 @@ double build_real_poly(const Params &p, const RealTable &t, RealPoly &f) {
   f.ta = (float)ta;
   f.tb = (float)tb;
   f.cg = (float)(p.xi * p.xi * 1.4426950408889634);
-  // sample points: table nodes from contact to r_cut, about 500 of them, the ends included
+  // sample points: table nodes from contact to r_cut, about 160 of them (16 per extremum of
+  // the error), the ends included
   std::vector<int> node;
   const int last = std::min(t.len - 1, (int)std::floor(rc / t.dr));
   if (last - t.k2 < 4 * NB) return HUGE_VAL;
-  const int step = std::max(1, (last - t.k2) / 500);
+  const int step = std::max(1, (last - t.k2) / 160);
   for (int i = t.k2; i < last; i += step) node.push_back(i);
   node.push_back(last);
   const int n = (int)node.size();
@@ -532,8 +533,12 @@ double build_real_poly(const Params &p, const RealTable &t, RealPoly &f) {
     // Lawson's iteration: least squares with weights that grow where the error is large
     // tends to the minimax fit; g weighs the error of P back to that of f
     std::fill(w.begin(), w.end(), 1.0);
-    double best = HUGE_VAL, cheb[NB] = {0};
+    double best = HUGE_VAL, before = HUGE_VAL, cheb[NB] = {0};
     for (int it = 0; it < 30; ++it) {
+      if (it % 6 == 0) {  // six more rounds only if the last six gained a hundredth
+        if (best > 0.99 * before) break;
+        before = best;
+      }
       double M[NB][NB + 1] = {};
       for (int q = 0; q < n; ++q) {
         const double *b = &B[(size_t)q * NB], wg = w[q] * g[q];
