@@ -1226,6 +1226,9 @@ pse_status autotune_impl(pse_ctx *c, const double *pos, int reps, pse_tuning *ou
   PSE_TRY(setup_config(c, (const double *)dpos, s));
   PSE_TRY(philox_w1(c, 1, 1, c->d_v[0], s));  // any dense vector will do
   pse_tuning t{};
+  // a captured step graph holds the lanes, tiles and tile arrays that change from here on, also
+  // when the tuning ends early
+  ++c->layout_version;
   // lanes per particle of the pair sum: the S -> E product of the GMRES loop plus the full product
   const int lanes[5] = {1, 4, 8, 16, 32};
   double best = INFINITY;
@@ -1287,7 +1290,6 @@ pse_status autotune_impl(pse_ctx *c, const double *pos, int reps, pse_tuning *ou
   }
   PSE_TRY(retile(c, cand[bi]));
   PSE_TRY(setup_config(c, (const double *)dpos, s));
-  ++c->layout_version;  // a captured step graph holds the old tiles and lanes
   for (int d = 0; d < 3; ++d) t.tile[d] = c->ps[0].tile[d];
   t.best_real_ms = best;
   t.best_wave_ms = bw;
