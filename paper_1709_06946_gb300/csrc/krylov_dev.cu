@@ -25,6 +25,8 @@
 // the while-node condition) so an iteration needs no host round trip.
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "device_common.cuh"
 #include "krylov_math.cuh"
 #include "pse_internal.cuh"
@@ -503,4 +505,77 @@ void kd_all_active(pse_ctx *c, cudaStream_t s) {
   k_all_active<<<sys_blocks(c), 128, 0, s>>>(c->nsys, c->d_active);
 }
 
+namespace {
+
+__global__ void k_scalars(int n, const double *x, double *rec, double *rt) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  rec[i] = recip(x[i]);
+  rt[i] = root(x[i]);
+}
+
+__global__ void __launch_bounds__(32) k_lz_solve(KDev k, int j) {
+  __shared__ double sm[LZ_ROWS * 35];
+  lz_solve(k, 0, j, threadIdx.x, sm);
+}
+
+}  // namespace
+
 }  // namespace pse
+
+// The device's scalar arithmetic and tridiagonal square root on host arrays (not on any
+// product's path: the library's own checks call them).
+extern "C" {
+
+// rec = recip(x), rt = root(x); 0, or 1 on a CUDA error.
+int pse_internal_device_scalars(int n, const double *x, double *rec, double *rt) {
+  const size_t b = sizeof(double) * (size_t)n;
+  double *d = nullptr;
+  if (n < 1 || cudaMalloc(&d, 3 * b) != cudaSuccess) return 1;
+  cudaError_t e = cudaMemcpy(d, x, b, cudaMemcpyHostToDevice);
+  pse::k_scalars<<<(n + 127) / 128, 128>>>(n, d, d + n, d + 2 * n);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpy(rec, d + n, b, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(rt, d + 2 * n, b, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e == cudaSuccess ? 0 : 1;
+}
+
+// c = T^{1/2} e1 as iteration m - 1 of the Lanczos kernel takes it (alpha[0..m), beta[0..m-1)):
+// 0, 2 when the eigensolver gave up, 1 on a CUDA error.
+int pse_internal_device_sqrt_e1(int m, const double *alpha, const double *beta, double *c) {
+  if (m < 1 || m > 120) return 1;
+  const size_t L = (size_t)m, nodes = 2 * pse::SQRT_NODES;
+  std::vector<double> h(pse::COEF_STRIDE + 4 * L + 1 + nodes + 2 * L + L * L + 1, 0.0);
+  double *p = nullptr;
+  if (cudaMalloc(&p, sizeof(double) * h.size()) != cudaSuccess) return 1;
+  pse::KDev k{};
+  k.nsys = 1;
+  k.lmax = m;
+  k.coef = p;
+  k.l_alpha = k.coef + pse::COEF_STRIDE;
+  k.l_beta = k.l_alpha + L;
+  k.l_cprev = k.l_beta + L;
+  k.l_c = k.l_cprev + L;
+  k.l_err = k.l_c + L;
+  k.l_nodes = k.l_err + 1;
+  k.l_work = k.l_err + 1 + nodes;
+  k.l_capped = (int *)(k.l_work + 2 * L + L * L);
+  h[pse::CO_H1 + m - 1] = alpha[m - 1];
+  for (int i = 0; i + 1 < m; ++i) {
+    h[pse::COEF_STRIDE + i] = alpha[i];
+    h[pse::COEF_STRIDE + L + i] = beta[i];
+  }
+  double *hn = &h[pse::COEF_STRIDE + 4 * L + 1];
+  pse::sqrt_nodes(pse::SQRT_NODES, pse::SQRT_WINDOW, hn, hn + pse::SQRT_NODES);
+  int capped = 0;
+  cudaError_t e = cudaMemcpy(p, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice);
+  pse::k_lz_solve<<<1, 32>>>(k, m - 1);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpy(c, k.l_c, sizeof(double) * L, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(&capped, k.l_capped, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(p);
+  return e != cudaSuccess ? 1 : (capped ? 2 : 0);
+}
+
+}  // extern "C"

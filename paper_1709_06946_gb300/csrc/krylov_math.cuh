@@ -127,10 +127,10 @@ inline void sqrt_nodes(int n, double window, double *s, double *w) {
   }
 }
 
-// 1 / d and sqrt(x) in FP64.  On the device, for arguments well inside the FP32 range, an
-// FP32 seed and Newton steps (each doubles the correct digits: 7, 14, 28): the FP64 unit
-// issues one warp instruction in sixteen cycles and the library forms are serial chains
-// of several tens of them.
+// 1 / d and sqrt(x) in FP64, to two units in the last place.  On the device, for arguments well
+// inside the FP32 range, an FP32 seed (7 digits) and two Newton steps (14, then FP64's
+// 16): the FP64 unit issues one warp instruction in sixteen cycles and the library forms
+// are serial chains of several tens of them.
 __host__ __device__ inline double recip(double d) {
 #ifdef __CUDA_ARCH__
   const float f = (float)d;
