@@ -328,7 +328,15 @@ def real_flops_per_pair():
     return {'full': 178, 'se': 130, 'fsu': 82, 'su': 68}
 
 
+PAIR_FLOPS_NOTE = ('operations of the formulas with tabulated functions in the Y basis over the time; the kernel '
+                   'evaluates polynomials in Cartesian components, so this is no utilisation of the FP32 units')
 EST_FLOPS_PER_PAIR = 250        # a-priori estimate of the full 8 x 8 block per pair direction
+
+
+def uses_tile_kernels(info):
+    """Whether a handle (its info) spreads and interpolates with the kernels for tiles of up to 16^3 points: they
+    also take grids that 16 does not divide (54 = 14 + 14 + 14 + 12), and not every 16^3 tiling (FP64)."""
+    return bool(info['tile_kernels'])
 
 
 def kernel_instances(prof, N, Ng, P, npairs, cubic, wave_kernel=0):
@@ -339,7 +347,7 @@ def kernel_instances(prof, N, Ng, P, npairs, cubic, wave_kernel=0):
     vm, vc = prof['variant_ms'], prof['variant_calls']
     n3 = Ng ** 3
     nkh = Ng * Ng * (Ng // 2 + 1)
-    # kernel names: 16^3 tiles take the grid-column spreading with the CTA-wide candidate scan and
+    # kernel names: tiles of up to 16^3 points take the grid-column spreading with the CTA-wide candidate scan and
     # the staged-region interpolation by default (wave_kernel bit 0: shared-tile spreading; bit 2:
     # column spreading with a scan per warp; bit 1: column, bit 4: tile-owned interpolation), other
     # tiles the general kernels
@@ -372,7 +380,7 @@ def kernel_instances(prof, N, Ng, P, npairs, cubic, wave_kernel=0):
             continue
         per = ms / calls / 1e3
         out.append({'kernel': 'k_real<float,%s>' % mode, 'stage': 'real', 'bound': 'alu', 'launches': calls,
-                    'ms': ms, 'us_per_launch': per * 1e6, 'flops_per_pair': fl[v],
+                    'ms': ms, 'us_per_launch': per * 1e6, 'flops_per_pair': fl[v], 'flops_note': PAIR_FLOPS_NOTE,
                     'algorithmic_flops_per_launch': npairs * fl[v],
                     'achieved': npairs * fl[v] / per / 1e12, 'unit': 'TFLOP/s'})
     return out
@@ -451,7 +459,7 @@ def run_ours(args, world, rank, local, pg):
     Ng, N = inf['Ng'], args.N
     n3 = Ng ** 3
     K = KP
-    cubic = tuple(inf['tile']) == (16, 16, 16)
+    cubic = uses_tile_kernels(inf)
     kernels = kernel_instances(prof, N, Ng, inf['P'], npairs, cubic, args.wave_kernel)
     traffic_ok = (args.N, args.phi, args.tol, args.xi, Ng, inf['P']) == NCU_TRAFFIC_WORKLOAD
     for k in kernels:
@@ -469,8 +477,8 @@ def run_ours(args, world, rank, local, pg):
                           'derived FP32 peak: 152 SMs x 128 lanes x 2 flop x 2070 MHz'),
             'per_launch': ('algorithmic bytes %.4g (per-particle and per-grid-point bytes x units)' %
                            dom['algorithmic_bytes_per_launch']) if dom['bound'] == 'hbm' else
-                          ('flops %.4g (%d per ordered pair x %.4g pairs)' %
-                           (dom['algorithmic_flops_per_launch'], dom['flops_per_pair'], npairs))}
+                          ('flops %.4g (%d per ordered pair x %.4g pairs): %s' %
+                           (dom['algorithmic_flops_per_launch'], dom['flops_per_pair'], npairs, PAIR_FLOPS_NOTE))}
     # the pair sum: all of its instances against the derived FP32 peak, with the formula flops per
     # pair and the a-priori ~250-flop estimate of the full block beside them
     fl = real_flops_per_pair()
@@ -480,7 +488,7 @@ def run_ours(args, world, rank, local, pg):
                  'peak': FP32_PEAK_TFLOPS_AT_MAX, 'unit': 'TFLOP/s',
                  'frac': real_rate / FP32_PEAK_TFLOPS_AT_MAX if real_rate else None,
                  'peak_note': 'derived FP32 peak: 152 SMs x 128 lanes x 2 flop x 2070 MHz',
-                 'flops_per_pair': fl, 'estimate_flops_per_pair_full': EST_FLOPS_PER_PAIR,
+                 'flops_per_pair': fl, 'flops_note': PAIR_FLOPS_NOTE, 'estimate_flops_per_pair_full': EST_FLOPS_PER_PAIR,
                  'achieved_at_estimate_flops': (npairs * EST_FLOPS_PER_PAIR * (Li + Ki + K)
                                               / (stage_ms['real'] / 1000.0) / 1e12) if stage_ms['real'] > 0 else None}
     # per-step algorithmic rates of the wave-space stages, and the ceiling that binds spreading and
