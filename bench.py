@@ -312,10 +312,10 @@ def accuracy_vs_fp64(pkg, torch, dev, args, pos_np, L, h64):
 # benchmark workload (N = 1048576, phi = 0.3, eps = 1e-3, xi = 0.5, N_g = 256, P = 6): ncu captures of
 # the N = 524288 case of the same workload (profiles/dram_bytes_N524288_phi0.3_eps1e-3.md), scaled to a
 # full launch by the ordered pairs (1.1017e8 / 5.5086e7): the pair sum's DRAM bytes are its neighbour
-# records.  The wave-space kernels are left out (their grid bytes stay partly in L2 between launches,
+# records and the rows that leave L2 between their readers.  The wave-space kernels are left out (their grid bytes stay partly in L2 between launches,
 # so they do not scale with N_g^3).  Reported only for that workload.
 NCU_TRAFFIC_WORKLOAD = (1048576, 0.3, 1e-3, 0.5, 256, 6)
-NCU_TRAFFIC = {'k_real<float,M_FULL>': 1.764e9, 'k_real<float,M_SE>': 1.739e9}
+NCU_TRAFFIC = {'k_real<float,M_FULL>': 2.016e9, 'k_real<float,M_SE>': 1.987e9}
 
 
 def real_flops_per_pair():

@@ -5,8 +5,8 @@
 // A handle holds one suspension (pse_create) or a group of independent
 // suspensions (pse_create_batch) that every kernel processes in one launch.
 // The Krylov iterations of the suspensions run in lockstep, each with its own
-// FP64 scalars on the host (Lanczos tridiagonal, GMRES Hessenberg and Givens
-// rotations); a suspension that has converged drops out of the launches.
+// FP64 scalars on the device (Lanczos tridiagonal, GMRES Hessenberg and Givens
+// rotations; krylov_dev.cu); a suspension that has converged drops out of the launches.
 // Vectors live on the device.
 #include <algorithm>
 #include <cmath>

@@ -172,7 +172,7 @@ __device__ __forceinline__ void pair_terms(const T rh[3], const T row[8], const 
 // components take about 60 operations (110 in the Y basis).  At 2^20 particles, 105
 // neighbours each: full product 886 -> 630 us, S -> E 648 -> 415, S -> U 594 -> 364;
 // FP64 form at 11000 particles 630 -> 445 us.  Below 10^5 particles the few thousand warps
-// wait on their records (47 us at 64000, 68 before).
+// wait on their records (S -> E at 64000 49 us, 67 before).
 //
 // FP32, polynomials: 48 registers so that five 256-thread CTAs fit an SM (four: S -> E 487
 // us; six: full 751 us, spilled).  With the table 64 registers and four, as its lookups of the

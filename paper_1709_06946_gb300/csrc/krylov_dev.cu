@@ -149,7 +149,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // 35 doubles): alpha_j, c_m = T_m^{1/2} e1 and the relative change of the iterate.  A block
 // of its own takes it beside the blocks that update w, and not their last one after
 // them; and loop control counts suspensions, not blocks: k_kr_finish at 50,000 particles
-// and ten iterations 21.4 -> 18.3 us per launch, at 3000 14.4 -> 11.8.
+// and ten iterations 23 -> 20 us per launch, at 3000 16 -> 14.
 __device__ void lz_solve(const KDev &k, int q, int j, int lane, double *sm) {
   const int m = j + 1, L = k.lmax;
   const double *cf = k.coef + (size_t)q * COEF_STRIDE, *be = k.l_beta + (size_t)q * L, *cp = k.l_cprev + (size_t)q * L;

@@ -113,7 +113,7 @@ struct SysDev {
   int64_t cgrid0, cstride; // half spectrum component c at cgrid0 + c * cstride (complex)
   int N, Ng, nkx, nc, slots, tile0, cell0, blk0;
   int T[3], nt[3];
-  int cubic;               // 1: mixed precision, P in {5, 6, 8}, 16^3 tiles, >= 2 tiles per side
+  int cubic;               // 1: the kernels for tiles of up to 16^3 points take it (set_cubic)
   double L, h, cs;
   double inv_h, inv_cs;    // 1/h and 1/cs (binning without FP64 divisions)
   float Lf, csf;

@@ -276,21 +276,20 @@ __device__ __forceinline__ unsigned region_mask(int ex, int ey, int ez, int wx, 
 // them.  Half a tile on a CTA of 8 warps against the whole tile on one of 16: the halves
 // even out the last wave (216 tiles at N_g = 96) and do not wait for each other at the
 // barriers, for a quarter more candidates scanned: 8 components at N_g = 36 15.1 -> 11.8
-// us, 5 components at N_g = 96 58.0 -> 53.3, at N_g = 256 (2^20 particles) 552 -> 519 and 8
-// components 950 -> 869.  Quarters (8 rows of y) take 11.3, 59.0, 582 and 962 us.
+// us, 5 components at N_g = 96 60 -> 57, at N_g = 256 (2^20 particles) 620 -> 590 and 8
+// components 950 -> 869.  Quarters (8 rows of y) take 11.3, 61, 654 and 962 us.
 //
 // Bound by instruction issue (62 % of the slots at N = 524288) and the barriers between
 // scan and update.  A record carries its support start as floats and a list
 // entry is the record's offset, so that a visit needs no integer to float conversion (the
-// quarter-rate unit of the exponential) and no multiplication for the address: 5 components
-// at P = 6, 2^20 particles 668 -> 549 us, 64,000 70 -> 58, 30,000 36 -> 30; P = 8,
-// 150,000 particles 155 -> 139.
+// quarter-rate unit of the exponential) and no multiplication for the address.  Both changes
+// together, median launch: 5 components at P = 6, 2^20 particles 657 -> 588 us, 64,000 63 ->
+// 56, 30,000 31 -> 26; 8 components, 2^20 1005 -> 876; P = 10, 150,000 353 -> 313.
 //
 // Tiles are 16^3 where 16 divides the grid, else as equal as possible (54 = 14 + 14 + 14 +
 // 12); columns and planes past a smaller tile's edge are idle.  Against the general
-// kernel: 5 components on 12^3 tiles at N_g = 36 65 -> 29 us (22 with the changes above), the 11-moment
-// product's 8 and 3 components at N_g = 128 322 -> 120 and 199 -> 71 us (103 and 61 with
-// the changes above).
+// kernel: 5 components on 12^3 tiles at N_g = 36 64 -> 25 us, the 11-moment product's 8
+// and 3 components at N_g = 128 324 -> 105 and 198 -> 59 us.
 template <int C, int SLOT0, int P, int ZT, bool DEF = false, int ROW = 8, int COMP0 = 0>
 __global__ void __launch_bounds__(32 * COLQ_WARPS, ZT < CUBE && C <= 5 ? 4 : 2)
     k_spread_colq(WaveArgs wa, int *queue, const int4 *__restrict__ sp_i0, const float4 *__restrict__ sp_d0,

@@ -11,8 +11,8 @@
 // l), walk each column along z, and the quarter sums its lanes with three
 // shuffles, so every output row is written by one lane with no atomic addition
 // (the tile-owned kernel splits a support over up to 8 tiles and adds the parts).
-// Against the general kernel on 12^3 tiles at N_g = 36: 5 components 55 -> 7.4 us, 8
-// components 39 -> 8.7; the 11-moment product's at N_g = 128 187 -> 105 and 133 -> 60 us.
+// Against the general kernel on 12^3 tiles at N_g = 36: 5 components 54 -> 8.1 us, 8
+// components 33 -> 7.7; the 11-moment product's at N_g = 128 188 -> 97 and 134 -> 50 us.
 // Two CTAs share an SM (about 83 KB each for 5 components, P = 6), so one CTA's
 // staging overlaps the other's read-out; where staging is most of the work an item is a whole
 // tile whose planes pass through a ring (halo_may_ring).

@@ -217,8 +217,8 @@ void interp_p(pse_ctx *c, const WaveArgs &a, void *vout, cudaStream_t s) {
 }  // namespace
 
 // mode selects the interpolated components: M_FULL U,E (8), M_SE E (5), M_FSU U (3)
-// Suspensions with 16^3 tiles: the shared-memory tile (default) or grid columns
-// in registers (bit 1 of option wave_kernel).
+// Suspensions with tiles of up to 16^3 points: the staged region (default), grid columns in
+// registers (bit 1 of option wave_kernel) or the shared-memory tile (bit 4).
 void interp_cubic(pse_ctx *c, const WaveArgs &a, void *vout, int mode, cudaStream_t s) {
   if (c->opt.wave_kernel & 2) interp_col_launch(c, a, vout, mode, s);
   else if (c->opt.wave_kernel & 16) interp16_launch(c, a, vout, mode, s);
