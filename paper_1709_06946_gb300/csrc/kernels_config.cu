@@ -493,45 +493,40 @@ __global__ void __launch_bounds__(NBR_NT, sizeof(T) == 4 ? 4 : 1)
 }
 
 // The same list, one thread per particle, for systems of mostly empty cells (use_sparse):
-// a thread streams through the cell-ordered records of its 25 runs, NB of them loaded before
+// a thread streams through the cell-ordered records of its runs, NB of them loaded before
 // the first is tested.  Bound by the latency of that walk; 10^6 particles at a volume fraction of
-// 0.01 take 165 us, 983 with a warp per cell.
-template <typename T, bool DEF>
-__global__ void __launch_bounds__(128)
-    k_nbr_sparse(const SysDev *__restrict__ sys, const int64_t *__restrict__ p0, int nsys, int64_t Ntot, float rc2f,
-                 double rc2, const typename V4<T>::t *__restrict__ rs_cell, const int4 *__restrict__ sp_i0,
-                 const int *__restrict__ cell_start, const int *__restrict__ cell_pos, int *cnt, typename V4<T>::t *geo,
-                 unsigned long long *tot, int *ovf) {
+// 0.01 take 177 us, 983 with a warp per cell.  Returns the particle's neighbour count; self: its own
+// cell-list position, packed: its cell.
+template <typename T, bool DEF, bool WIDE>
+__device__ __forceinline__ int nbr_particle(const SysDev &a, int self, int packed, T r2max,
+                                            const typename V4<T>::t *__restrict__ rs_cell,
+                                            const int *__restrict__ cell_start, typename V4<T>::t *row_geo) {
   using T4 = typename V4<T>::t;
-  constexpr int NB = 4;  // candidate records loaded before the first is tested
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= Ntot) return;
-  const int si = find_sys(p0, nsys, i), self = cell_pos[i], packed = sp_i0[i].w;
-  const SysDev &a = sys[si];
+  constexpr int NB = 4;
   const int nc = a.nc, slots = a.slots, cell0 = a.cell0;
   const T cs = sizeof(T) == 4 ? (T)a.csf : (T)a.cs, L = sizeof(T) == 4 ? (T)a.Lf : (T)a.L;
-  const T r2max = sizeof(T) == 4 ? (T)rc2f : (T)rc2;
   T A[DEF ? 9 : 1];
   if constexpr (DEF) {
 #pragma unroll
     for (int m = 0; m < 9; ++m) A[m] = sizeof(T) == 4 ? (T)a.Af[m] : (T)a.A[m];
   }
   const int cx = packed & 1023, cy = (packed >> 10) & 1023, cz = packed >> 20;
+  const int span = WIDE ? 5 : nc, y0 = WIDE ? cy - 2 : 0, z0 = WIDE ? cz - 2 : 0;
+  const int x0 = WIDE ? cx - 2 : 0, x1 = WIDE ? cx + 2 : nc - 1;
   const T4 own = rs_cell[self];
   const T ctr[3] = {own.x, own.y, own.z};
-  T4 *row_geo = geo + a.nbr0 + (i - a.p0) * slots;
   int n = 0;
-  for (int dz = -2; dz <= 2; ++dz)
-    for (int dy = -2; dy <= 2; ++dy) {
-      const int rz = cz + dz, ry = cy + dy;
+  for (int iz = 0; iz < span; ++iz)
+    for (int iy = 0; iy < span; ++iy) {
+      const int rz = z0 + iz, ry = y0 + iy;
       const int wz = rz < 0 ? -1 : (rz >= nc ? 1 : 0), wy = ry < 0 ? -1 : (ry >= nc ? 1 : 0);
       const int row = cell0 + ((rz - wz * nc) * nc + (ry - wy * nc)) * nc;
-      const T sy = sizeof(T) == 4 ? (T)-dy : (T)wy, sz = sizeof(T) == 4 ? (T)-dz : (T)wz;
-      // cells [cx - 2, cx + 2], in two ranges where they wrap
-      for (int wx = cx < 2 ? -1 : 0; wx <= (cx + 2 >= nc ? 1 : 0); ++wx) {
-        const int kb = cell_start[row + max(cx - 2 - wx * nc, 0)];
-        const int ke = cell_start[row + min(cx + 2 - wx * nc, nc - 1) + 1];
-        const T sx = sizeof(T) == 4 ? (T)(cx - wx * nc) : (T)wx;
+      const T sy = sizeof(T) == 4 ? (T)(WIDE ? 2 - iy : cell_offset(cy - ry, nc)) : (T)wy;
+      const T sz = sizeof(T) == 4 ? (T)(WIDE ? 2 - iz : cell_offset(cz - rz, nc)) : (T)wz;
+      // cells [x0, x1], in two ranges where they wrap
+      for (int wx = x0 < 0 ? -1 : 0; wx <= (x1 >= nc ? 1 : 0); ++wx) {
+        const int kb = cell_start[row + max(x0 - wx * nc, 0)];
+        const int ke = cell_start[row + min(x1 - wx * nc, nc - 1) + 1];
         for (int k = kb; k < ke; k += NB) {
           T4 q[NB];
 #pragma unroll
@@ -540,7 +535,9 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
           for (int u = 0; u < NB; ++u) {
             if (k + u >= ke) break;
-            T4 rec = nbr_sep<T, DEF, true>(ctr, q[u], sizeof(T) == 4 ? sx - (T)q[u].w : sx, sy, sz, cs, L, A);
+            T sx = (T)wx;
+            if (sizeof(T) == 4) sx = WIDE ? (T)(cx - wx * nc) - (T)q[u].w : (T)cell_offset(cx - (int)q[u].w, nc);
+            T4 rec = nbr_sep<T, DEF, WIDE>(ctr, q[u], sx, sy, sz, cs, L, A);
             if (rec.x * rec.x + rec.y * rec.y + rec.z * rec.z < r2max && k + u != self) {
               if (n < slots) {
                 rec.w = index_as_real<T>(k + u);
@@ -552,8 +549,25 @@ __global__ void __launch_bounds__(128)
         }
       }
     }
+  return n;
+}
+
+template <typename T, bool DEF>
+__global__ void __launch_bounds__(128)
+    k_nbr_sparse(const SysDev *__restrict__ sys, const int64_t *__restrict__ p0, int nsys, int64_t Ntot, float rc2f,
+                 double rc2, const typename V4<T>::t *__restrict__ rs_cell, const int4 *__restrict__ sp_i0,
+                 const int *__restrict__ cell_start, const int *__restrict__ cell_pos, int *cnt, typename V4<T>::t *geo,
+                 unsigned long long *tot, int *ovf) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= Ntot) return;
+  const int si = find_sys(p0, nsys, i), self = cell_pos[i], packed = sp_i0[i].w;
+  const SysDev &a = sys[si];
+  const T r2max = sizeof(T) == 4 ? (T)rc2f : (T)rc2;
+  typename V4<T>::t *row_geo = geo + a.nbr0 + (i - a.p0) * a.slots;
+  const int n = a.nc >= 5 ? nbr_particle<T, DEF, true>(a, self, packed, r2max, rs_cell, cell_start, row_geo)
+                          : nbr_particle<T, DEF, false>(a, self, packed, r2max, rs_cell, cell_start, row_geo);
   cnt[i] = n;
-  if (n > slots) atomicOr(ovf, 1);
+  if (n > a.slots) atomicOr(ovf, 1);
   // one atomic addition per warp when its particles share a suspension
   const unsigned act = __activemask();
   const int leader = __ffs(act) - 1;
@@ -577,13 +591,11 @@ void *alloc_dev(pse_ctx *c, size_t bytes) {
 // has few candidates for its lanes and few particles to test them against, and walks past
 // the empty cells one after the other.  A thread's serial walk over 25 runs takes 20 us and more,
 // so there have to be many cells for it (600 per SM).  Measured, us, warp / thread:
-//   FP32  N = 10^6: 0.1 particles per cell 983 / 165, 0.86 708 / 348, 1.5 756 / 535, 2.2 860 / 734
-//         300000: 0.02 850 / 53, 0.87 230 / 133, 1.5 243 / 204, 2.1 265 / 263;  200000: 1.5 167 / 163, 1.8 174 / 205
+//   FP32  N = 10^6: 0.1 particles per cell 983 / 177, 0.86 708 / 346, 1.5 756 / 535, 2.2 860 / 734
+//         300000: 0.02 850 / 63, 0.87 230 / 132, 1.5 243 / 204, 2.1 265 / 263;  200000: 1.5 167 / 163, 1.8 174 / 205
 //         60000: 0.22 61 / 31, 0.87 55 / 51, 1.3 56 / 65;  30000: 0.11 44 / 26, 0.44 33 / 38;  10000: 0.11 21 / 23
 //   FP64  300000: 0.11 477 / 489, 0.21 435 / 686;  100000: 0.02 499 / 103;  30000: 0.02 164 / 42, 0.11 74 / 81
 bool use_sparse(const pse_ctx *c) {
-  for (const Params &p : c->ps)
-    if (p.nc < 5) return false;
   if (c->ncells < 600 * (int64_t)c->nsm) return false;
   return c->prec == PSE_MIXED ? 2 * c->ncells >= c->p.N + 65536 : c->ncells >= 16 * c->p.N;
 }

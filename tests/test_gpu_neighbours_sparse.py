@@ -87,3 +87,11 @@ def test_dilute_suspensions(pkg, prec):
     Ls = [0.5 * RC * (nc + 0.01) for nc in (40, 5, 36)]
     pos = [_corner(n, L, n) for n, L in zip((300, 1, 173), Ls)]
     assert _check(pkg, pos, Ls, prec) >= 91200
+
+
+@pytest.mark.parametrize('prec', ['fp64', 'mixed'])
+def test_few_cells_beside_dilute_suspensions(pkg, prec):
+    """Four cells per side (every cell once, nearest image by rounding) and five in the same launch."""
+    Ls = [0.5 * RC * (nc + 0.01) for nc in (46, 4, 5)]
+    pos = [_corner(260, Ls[0], 260)] + [pse_inputs.rsa_positions(n, 0.0, seed=n, L=L)[0] for n, L in zip((50, 60), Ls[1:])]
+    assert _check(pkg, pos, Ls, prec) >= 91200
